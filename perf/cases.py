@@ -122,15 +122,25 @@ def _out_dims(c):
     return (c["H"] - c["Fh"]) // c["stride"] + 1, (c["W"] - c["Fw"]) // c["stride"] + 1
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """N(0,1) values inside an explicit zero ring of `pad`; Kaiming-normal filters (none for the transform)."""
     dev = torch.device("cuda")
     gen = torch.Generator(device=dev).manual_seed(seed)
-    N, C, H, W, K, Fh, Fw, _ = dims = _dims(case)
-    Ho, Wo = _out_dims(case)
-    op, mode, p = case["op"], MODES[case["mode"]], case["pad"]
-    # N(0,1) values inside an explicit zero ring of `pad`; Kaiming-normal filters
+    N, C, H, W, K, Fh, Fw, _ = _dims(case)
+    p = case["pad"]
     x = torch.zeros((N, C, H, W), device=dev)
     x[:, :, p:H - p, p:W - p].normal_(generator=gen)
+    if case["op"] == "transform":
+        return x, None
+    return x, torch.empty((K, C, Fh, Fw), device=dev).normal_(generator=gen) * math.sqrt(2.0 / (C * Fh * Fw))
+
+
+def prepare(case, seed):
+    dev = torch.device("cuda")
+    N, C, H, W, K, Fh, Fw, _ = dims = _dims(case)
+    Ho, Wo = _out_dims(case)
+    op, mode = case["op"], MODES[case["mode"]]
+    x, f = _inputs(case, seed)
     st = {"op": op, "mode": mode, "dims": dims, "x": x}
     if op in ("transform", "im2win"):
         st["xhat"] = torch.empty((N, C, Ho, W * Fh), device=dev)
@@ -138,7 +148,7 @@ def prepare(case, seed):
         st["xhat"] = torch.empty((N, C, Ho, W * Fh), device=dev, dtype=torch.bfloat16)
     if op == "transform":
         return st
-    st["f"] = torch.empty((K, C, Fh, Fw), device=dev).normal_(generator=gen) * math.sqrt(2.0 / (C * Fh * Fw))
+    st["f"] = f
     st["out"] = torch.empty((N, Ho, Wo, K) if op == "nhwc" else (N, K, Ho, Wo), device=dev)
     # The workspace with which the fastest kernels apply; the fused calls get what the unfused call would want,
     # so that shapes without a fused kernel are served too.
@@ -174,6 +184,36 @@ def run(st):
     b.transform_bf16(st["x"], dims, st["xhat"])
     b.conv(st["xhat"], b.SRC_IM2WIN_BF16, f, dims, mode, out, ws)
     return out, st["xhat"]
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits: the im2win tensor is a copy of input elements (rounded to bf16 where it is
+    stored so), the convolution Eq. 1 as one matrix product per image."""
+    N, C, H, W, K, Fh, Fw, s = _dims(case)
+    Ho, Wo = _out_dims(case)
+    op = case["op"]
+    x, f = _inputs(case, seed)
+    xhat = None
+    if op in ("transform", "conv", "im2win", "im2win_bf16"):  # Ihat[i][r][m][k*Fh+u] = I[i][r][m*s+u][k]
+        xhat = torch.empty((N, C, Ho, W, Fh), device=x.device)
+        for u in range(Fh):
+            xhat[..., u] = x[:, :, u:u + (Ho - 1) * s + 1:s]
+        xhat = xhat.view(N, C, Ho, W * Fh)
+        if op == "transform":
+            return xhat
+        if op == "im2win_bf16":
+            xhat = xhat.bfloat16()
+        if op == "conv":
+            xhat = xhat.view(-1)
+    f64 = f.double().view(K, C * Fh * Fw)
+    out = torch.empty((N, K, Ho * Wo), device=x.device, dtype=torch.float64)
+    for i in range(N):
+        cols = torch.nn.functional.unfold(x[i:i + 1].double(), (Fh, Fw), stride=s)[0]
+        torch.mm(f64, cols, out=out[i])
+    out = out.view(N, K, Ho, Wo)
+    if op == "nhwc":
+        return out.permute(0, 2, 3, 1).contiguous()
+    return out if op == "fused" else (out, xhat)
 
 
 def work(case):
