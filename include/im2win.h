@@ -77,8 +77,9 @@ int im2win_workspace_bytes(const im2win_shape* shape, size_t* bytes);
 /* Workspace with which im2win_conv can pick its fastest kernel for (shape, src_kind, mode) (no
  * counterpart in the paper): the im2win tensor where src_kind is NCHW (as above, rounded up to 256
  * bytes), plus room for a re-laid-out copy of the filter that some tensor-core kernels stream by TMA
- * (tap-major orders for the strip-matrix and window-offset kernels; bf16 for BF16 mode).  That copy is at
- * most about 1.4 x the filter's own 4*K*C*Fh*Fw bytes, i.e. a few MB against an im2win tensor of tens to hundreds
+ * (tap-major orders for the strip-matrix and window-offset kernels; bf16 for BF16 mode; rows padded to whole
+ * channel groups where C is odd).  That copy is at most about 1.4 x the filter's own 4*K*C*Fh*Fw bytes (with
+ * fewer than 16 channels: those of a filter of 16), i.e. a few MB against an im2win tensor of tens to hundreds
  * of MB.  A smaller workspace is legal (down to im2win_workspace_bytes, or none for the other source
  * kinds): kernels that need no copy are used instead, some of them slower. */
 int im2win_conv_workspace_bytes(const im2win_shape* shape, int src_kind, int mode, size_t* bytes);
@@ -116,7 +117,8 @@ int im2win_transform_bf16(const float* in_nchw, const im2win_shape* shape, uint1
  *            needs and reads the windows from them, so nothing of size Ihat is written (workspace
  *            0 bytes).  Same result as the other two kinds.  Shapes without a fused specialisation
  *            (the specialised filter sizes are 3x3, 5x5, 7x7, 11x11 and, with channel counts that are
- *            multiples of 16, 1x1, 1x3, 3x1, 1x7, 7x1, 2x2, 4x4, 3x5, 5x3) fall back to transform + convolution if a
+ *            multiples of 16, 1x1, 1x3, 3x1, 1x7, 7x1, 2x2, 4x4, 3x5, 5x3) fall back to transform + convolution (other
+ *            channel counts of these filter sizes: to the fused kernel with a padded last channel group) if a
  *            sufficient `workspace` is given, else EUNSUPPORTED; IM2WIN_MODE_FP32 always takes that
  *            fallback.
  *            src_kind IM2WIN_BF16: a bf16 im2win tensor from im2win_transform_bf16; mode must be

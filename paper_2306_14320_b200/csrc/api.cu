@@ -246,6 +246,9 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
     Scratch sc;
     offset = (offset + 255) / 256 * 256;
     if (ws_bytes > offset) { sc.ptr = ws + offset; sc.bytes = ws_bytes - offset; }
+    // (an im2win tensor at hand, or room for one: the generic kernel could take the call)
+    sc.wide = !out16 && (src_kind == IM2WIN_SRC_IM2WIN || src_kind == IM2WIN_SRC_NCHW ||
+                         (src_kind == IM2WIN_SRC_NCHW_FUSED && ws_bytes >= win_bytes));
     return sc;
   };
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);

@@ -52,6 +52,7 @@ int launch_conv_fp32(const float* xhat, const float* f, float* out, const Geomet
 struct Scratch {
   void* ptr = nullptr;
   size_t bytes = 0;
+  bool wide = false;  // the generic kernel could serve the call: specialisations may take shapes beyond their documented lists
 };
 // Tensor-core convolution kernels.  Each returns IM2WIN_EUNSUPPORTED when it does not apply (shape,
 // scratch) before anything is enqueued; launch_conv_tc tries them in order of expected speed.
