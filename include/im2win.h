@@ -166,7 +166,7 @@ int im2win_conv_nhwc(const void* src, int src_kind, const float* filter_kcfhfw,
  * element: half the output footprint and half the bytes written.
  * out_nchw_bf16: device, N*K*Ho*Wo 16-bit words, every element is written; 16-byte aligned.
  * Everything else as im2win_conv.  Tensor-core modes only (IM2WIN_MODE_FP32: EINVAL), and only
- * square filters with a specialisation: 3x3, 5x5, 7x7, 11x11 (EUNSUPPORTED otherwise: the generic
+ * square filters with a specialisation: 3x3, 5x5, 7x7, 11x11 (EUNSUPPORTED otherwise: the general
  * kernel and the pointwise / factorised families have no bf16 epilogue). */
 int im2win_conv_bf16out(const void* src, int src_kind, const float* filter_kcfhfw,
                         const im2win_shape* shape, int mode, uint16_t* out_nchw_bf16,

@@ -150,7 +150,7 @@ def workspace_bytes(shape) -> int:
     return b.value
 
 
-KERNEL_STRIP, KERNEL_PERSISTENT, KERNEL_GENERIC, KERNEL_FP32, KERNEL_WINDOW = 1, 2, 3, 4, 5
+KERNEL_STRIP, KERNEL_PERSISTENT, KERNEL_FP32, KERNEL_WINDOW, KERNEL_GATHER = 1, 2, 4, 5, 6
 
 
 def last_kernel() -> int:

@@ -65,7 +65,7 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
                    Scratch scratch, int src_kind, bool out_bf16) {
   // src_kind: 0 = fp32 im2win tensor, 1 = untransformed input consumed fused, 2 = bf16 im2win tensor.
   // Order: the window-offset and the strip-matrix kernel where each is implemented and expected to win, else
-  // the persistent specialised kernel, else (fp32 im2win tensor and fp32 output only) the generic kernel.
+  // the persistent specialised kernel.  (Where none applies, the caller takes the general kernel.)
   int rc = IM2WIN_EUNSUPPORTED;
   if (!knobs().force_generic) {
     rc = launch_conv_tc_window(src, f, out, g, mode, st, scratch, src_kind, out_bf16);
@@ -74,7 +74,7 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
     if (rc != IM2WIN_EUNSUPPORTED) return rc;
     rc = launch_conv_tc_persistent(src, f, out, g, mode, st, scratch, src_kind == 1, src_kind == 2, out_bf16);
     if (rc != IM2WIN_EUNSUPPORTED) return rc;
-    // sources the generic kernel does not read (bf16 im2win tensor, fused): the strip-matrix or the
+    // sources the general kernel does not read (bf16 im2win tensor, fused): the strip-matrix or the
     // window-offset kernel wherever one applies
     if (src_kind != 0 && !knobs().no_strip) {
       rc = launch_conv_tc_strip(src, f, out, g, mode, st, scratch, src_kind, out_bf16, /*even_if_slower=*/true);
@@ -85,8 +85,7 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
       if (rc != IM2WIN_EUNSUPPORTED) return rc;
     }
   }
-  if (src_kind != 0 || out_bf16) return IM2WIN_EUNSUPPORTED;
-  return launch_conv_tc_generic(static_cast<const float*>(src), f, out, g, mode, st);
+  return IM2WIN_EUNSUPPORTED;
 }
 
 size_t conv_scratch_bytes(const Geometry& g, int mode, int src_kind) {
@@ -246,18 +245,28 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
     Scratch sc;
     offset = (offset + 255) / 256 * 256;
     if (ws_bytes > offset) { sc.ptr = ws + offset; sc.bytes = ws_bytes - offset; }
-    // (an im2win tensor at hand, or room for one: the generic kernel could take the call)
+    // (an im2win tensor at hand, or room for one: the general kernel could take the call)
     sc.wide = !out16 && (src_kind == IM2WIN_SRC_IM2WIN || src_kind == IM2WIN_SRC_NCHW ||
                          (src_kind == IM2WIN_SRC_NCHW_FUSED && ws_bytes >= win_bytes));
     return sc;
   };
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  if (src_kind == IM2WIN_SRC_IM2WIN_BF16) {  // (no generic-kernel fallback for this storage variant)
+  if (src_kind == IM2WIN_SRC_IM2WIN_BF16) {  // (no general fallback for this storage variant)
     if (knobs().force_generic) return IM2WIN_EUNSUPPORTED;
     return launch_conv_tc(src, filter, out_nchw, g, mode, st, scratch_from(0), 2, out16);
   }
   const float* xhat = static_cast<const float*>(src);
+  // The general (gather) kernel reads the untransformed input as well as the im2win tensor: from SRC_NCHW it takes the
+  // former, so that it can overlap the transform (whose result the caller gets all the same).
+  const bool general = mode != IM2WIN_MODE_FP32 && !out16;
+  const bool from_input = src_kind != IM2WIN_SRC_IM2WIN;
+  const bool general_first = general && (knobs().force_generic || gather_preferred(g, mode, from_input));
   if (src_kind == IM2WIN_SRC_NCHW_FUSED) {
+    // (without room for the im2win tensor, shapes without a fused specialisation are refused: only these are tried)
+    if (general_first && ws_bytes >= win_bytes) {
+      rc = launch_conv_tc_gather(xhat, filter, out_nchw, g, mode, st, /*fused=*/true, /*behind_transform=*/false);
+      if (rc != IM2WIN_EUNSUPPORTED) return rc;
+    }
     if (mode != IM2WIN_MODE_FP32 && !knobs().force_generic) {
       rc = launch_conv_tc_window(xhat, filter, out_nchw, g, mode, st, scratch_from(0), 1, out16);
       if (rc == IM2WIN_EUNSUPPORTED && !knobs().no_strip)
@@ -271,8 +280,10 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
         rc = launch_conv_tc_window(xhat, filter, out_nchw, g, mode, st, scratch_from(0), 1, out16, /*even_if_slower=*/true);
       if (rc != IM2WIN_EUNSUPPORTED) return rc;
     }
-    // no fused kernel for this shape or mode: the unfused path, if the caller supplied a workspace
+    // no fused specialisation for this shape or mode: the general kernel or (fp32, bf16 output) the unfused path, if
+    // the caller supplied the workspace it takes
     if (ws_bytes < win_bytes) return IM2WIN_EUNSUPPORTED;
+    if (general) return launch_conv_tc_gather(xhat, filter, out_nchw, g, mode, st, /*fused=*/true, /*behind_transform=*/false);
     src_kind = IM2WIN_SRC_NCHW;
   }
   Scratch scratch = scratch_from(0);
@@ -283,7 +294,14 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
     scratch = scratch_from(win_bytes);
   }
   if (mode == IM2WIN_MODE_FP32) return launch_conv_fp32(xhat, filter, out_nchw, g, st);
-  return launch_conv_tc(xhat, filter, out_nchw, g, mode, st, scratch, 0, out16);
+  auto take_general = [&]() {
+    return launch_conv_tc_gather(from_input ? static_cast<const float*>(src) : xhat, filter, out_nchw, g, mode, st,
+                                 /*fused=*/from_input, /*behind_transform=*/from_input);
+  };
+  rc = general_first ? take_general() : IM2WIN_EUNSUPPORTED;
+  if (rc == IM2WIN_EUNSUPPORTED && !knobs().force_generic) rc = launch_conv_tc(xhat, filter, out_nchw, g, mode, st, scratch, 0, out16);
+  if (rc == IM2WIN_EUNSUPPORTED && general && !general_first) rc = take_general();
+  return rc;
 }
 
 }  // namespace im2win
@@ -357,7 +375,7 @@ int im2win_debug_set_option(const char* name, int value) {
       {"ntiles", &Knobs::ntiles}, {"transform_gather", &Knobs::transform_gather},
       {"test_skip_copy", &Knobs::test_skip_copy}, {"strip_mh", &Knobs::strip_mh}, {"strip_pair", &Knobs::strip_pair},
       {"force_window", &Knobs::force_window}, {"no_window", &Knobs::no_window}, {"window_mh", &Knobs::window_mh},
-      {"window_plan", &Knobs::window_plan}, {"window_pair", &Knobs::window_pair}, {"window_two", &Knobs::window_two}, {"window_nohelp", &Knobs::window_nohelp}, {"window_bres", &Knobs::window_bres}, {"transform_budget_kb", &Knobs::transform_budget_kb}};
+      {"window_plan", &Knobs::window_plan}, {"window_pair", &Knobs::window_pair}, {"window_two", &Knobs::window_two}, {"no_gather", &Knobs::no_gather}, {"gather_nt", &Knobs::gather_nt}, {"gather_z", &Knobs::gather_z}, {"gather_big", &Knobs::gather_big}, {"window_nohelp", &Knobs::window_nohelp}, {"window_bres", &Knobs::window_bres}, {"transform_budget_kb", &Knobs::transform_budget_kb}};
   for (const Entry& e : table)
     if (strcmp(e.name, name) == 0) { g_knobs.*(e.field) = value; return IM2WIN_OK; }
   return IM2WIN_EINVAL;

@@ -52,10 +52,10 @@ int launch_conv_fp32(const float* xhat, const float* f, float* out, const Geomet
 struct Scratch {
   void* ptr = nullptr;
   size_t bytes = 0;
-  bool wide = false;  // the generic kernel could serve the call: specialisations may take shapes beyond their documented lists
+  bool wide = false;  // the general (gather) kernel could serve the call: specialisations may take shapes beyond their documented lists
 };
 // Tensor-core convolution kernels.  Each returns IM2WIN_EUNSUPPORTED when it does not apply (shape,
-// scratch) before anything is enqueued; launch_conv_tc tries them in order of expected speed.
+// scratch) before anything is enqueued; launch_conv_tc tries the specialised ones in order of expected speed.
 // src_kind: 0 = fp32 im2win tensor, 1 = untransformed input consumed fused, 2 = bf16 im2win tensor.
 // (even_if_slower: take the problem wherever the kernel is implemented, not only where it is expected to
 // be the fastest -- for sources no other kernel accepts)
@@ -64,8 +64,6 @@ int launch_conv_tc_strip(const void* src, const float* f, float* out, const Geom
 int launch_conv_tc_persistent(const void* src, const float* f, float* out, const Geometry& g, int mode,
                               cudaStream_t st, Scratch scratch, bool fused = false, bool src_bf16 = false,
                               bool out_bf16 = false);
-int launch_conv_tc_generic(const float* xhat, const float* f, float* out, const Geometry& g, int mode,
-                           cudaStream_t st);
 int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                    Scratch scratch, int src_kind, bool out_bf16);
 // Scratch bytes with which every kernel above is available for this problem (0 if none wants any).
@@ -75,6 +73,11 @@ int launch_conv_tc_window(const void* src, const float* f, float* out, const Geo
                           Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower = false);
 size_t window_scratch_bytes(const Geometry& g, int mode, int src_kind);
 size_t persistent_scratch_bytes(const Geometry& g, int mode);
+// The gather kernel (conv_tc_gather.cu): fp32 sources (`fused`: the untransformed input), any filter size, fp32 output,
+// no scratch.  behind_transform: what this call has enqueued before is its own transform, which it may overlap.
+bool gather_preferred(const Geometry& g, int mode, bool fused);
+int launch_conv_tc_gather(const float* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
+                          bool fused, bool behind_transform);
 size_t conv_scratch_bytes(const Geometry& g, int mode, int src_kind);
 // Shared body of im2win_conv / im2win_conv_bf16out / im2win_conv_static (argument checks, workspace
 // split into the im2win tensor and the filter scratch, transform, dispatch).
@@ -88,7 +91,7 @@ inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? IM2WIN_OK : IM
 // linked into libim2win_test.so) keeps a mutable copy and exports im2win_debug_set_option(name, value)
 // to set a field by name, which is how the parity tests force each kernel configuration.
 struct Knobs {
-  int force_generic = 0;     // every tensor-core convolution through the generic kernel
+  int force_generic = 0;     // every tensor-core convolution through the general (gather) kernel, conv_tc_gather.cu
   int no_strip = 0;          // never use the strip-matrix kernel (conv_tc_strip.cu)
   int force_strip = 0;       // use the strip-matrix kernel wherever it is implemented, not only where its cost model picks it
   int no_box = 0;            // persistent kernel: strips by bulk copies instead of 2-D TMA boxes
@@ -113,13 +116,17 @@ struct Knobs {
   int window_pair = 0;       // window-offset kernel: 1 = CTA pairs forced, 2 = single CTAs forced, 0 = own choice
   int window_bres = 0;       // window-offset kernel: 1 = resident filter or nothing, 2 = never resident, 0 = own choice
   int window_nohelp = 0;     // window-offset kernel: the interleaver warps never help the epilogue
+  int no_gather = 0;         // gather kernel only where no other kernel applies
+  int gather_nt = 0;         // gather kernel: forced filter tile width (0: own choice)
+  int gather_z = 0;          // gather kernel: forced number of reduction slices (0: own choice)
+  int gather_big = 0;        // gather kernel: 64-bit indices
   int window_two = 0;        // window-offset kernel: 1 = two MMA-issuing threads forced, 2 = one forced, 0 = own choice
 };
 const Knobs& knobs();
 
 // Which convolution kernel the last launch on this host thread's library image used (a diagnostic the
 // test build exposes as im2win_debug_last_kernel; the product library only writes it).
-enum : int { KERNEL_NONE = 0, KERNEL_STRIP = 1, KERNEL_PERSISTENT = 2, KERNEL_GENERIC = 3, KERNEL_FP32 = 4, KERNEL_WINDOW = 5 };
+enum : int { KERNEL_NONE = 0, KERNEL_STRIP = 1, KERNEL_PERSISTENT = 2, KERNEL_FP32 = 4, KERNEL_WINDOW = 5, KERNEL_GATHER = 6 };
 void note_kernel(int which);
 // The launch plan of the last strip-matrix / window-offset launch (same diagnostic): up to eight integers.
 void note_plan(const int* v, int n);

@@ -1,6 +1,6 @@
 // im2win-based convolution (Algorithm 2) on the sm_100a tensor cores: persistent, specialised kernel.
 //
-// Same GEMM view as the generic kernel (M = output positions, N = filters, K = (r,u,v); A = windows in
+// GEMM view (M = output positions, N = filters, K = (r,u,v); A = windows in
 // TENSOR MEMORY written by tcgen05.st, B = filters in shared memory, fp32 accumulators in TMEM), with
 //   * one persistent CTA per SM walking work units t, t+grid, ... (neighbouring CTAs work on
 //     neighbouring tiles at the same time, so the few strip floats two tiles share are L2 hits);
@@ -1574,7 +1574,7 @@ int launch_spec_wide(const void* src, const float* f, float* out, const Geometry
 
 }  // namespace
 
-// Returns IM2WIN_EUNSUPPORTED when no specialisation applies (the caller then uses the generic kernel).
+// Returns IM2WIN_EUNSUPPORTED when no specialisation applies (the caller then uses the general kernel).
 // scratch: device memory of the caller's (beyond the im2win tensor) for the bf16 copy of a filter that
 // is too large to stay in shared memory (BF16 mode); without it those shapes are declined.
 // fused: `xhat` is the untransformed NCHW input and the windows are built from staged input rows
@@ -1654,7 +1654,7 @@ int launch_spec_11x11(IM2WIN_SPEC_ARGS) {
 
 // Pointwise, factorised, patch and other small rectangular filters (1x1; 1x3 / 3x1; 1x7 / 7x1; 2x2, 4x4; 3x5 / 5x3):
 // the same kernel, from the fp32 im2win tensor or
-// fused, fp32 NCHW or NHWC output (the bf16 storage variants of these shapes go to the generic kernel).
+// fused, fp32 NCHW or NHWC output (the bf16 storage variants of these shapes are refused).
 // Sixteen channels per group (TF32: two to six MMA steps, BF16: one to seven, no padding); 1x7 / 7x1 in TF32
 // mode: eight (seven steps).
 template <int FH, int FW>
@@ -1741,8 +1741,8 @@ int launch_conv_tc_persistent(const void* xhat, const float* f, float* out, cons
   const bool bf16 = mode == IM2WIN_MODE_BF16;
   const int rc = launch_family(xhat, f, out, g, st, scratch, kind, out_bf16, bf16, /*wide=*/false);
   // Channel counts that the families' groups do not divide: the last group's missing channels are zeros.  Taken
-  // where the generic kernel could serve the call too (what is refused without it stays refused), 3-15 x faster
-  // than that kernel (B200, whole calls: 3x5, C = 40, K = 72, 16 images of 45x61, BF16 199 -> 22.5 us; 3x3, C = 401,
+  // where the general kernel could serve the call too (what is refused without it stays refused), 3-15 x faster
+  // than without specialisation (B200, whole calls: 3x5, C = 40, K = 72, 16 images of 45x61, BF16 199 -> 22.5 us; 3x3, C = 401,
   // K = 32, one 43x43 image, TF32 334 -> 23 us; 1x1, C = 29, K = 64, 85 images of 27x36, BF16 64 -> 11.3 us).
   if (rc != IM2WIN_EUNSUPPORTED || !scratch.wide || kind == 2 || out_bf16) return rc;
   return launch_family(xhat, f, out, g, st, scratch, kind, out_bf16, bf16, /*wide=*/true);

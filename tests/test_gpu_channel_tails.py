@@ -6,7 +6,7 @@ import pytest
 
 from paper_2306_14320_b200 import binding as b
 from paper_2306_14320_b200 import workloads as wl
-from gpu_helpers import ensure_built, gpu_conv, oracle_conv, reset_config
+from gpu_helpers import apply_config, ensure_built, gpu_conv, oracle_conv, reset_config
 from test_gpu_nhwc import gpu_conv_nhwc
 
 torch = pytest.importorskip("torch")
@@ -36,14 +36,13 @@ def test_odd_channel_counts_bit_exact(dims, mode):
     f = wl.small_ints(32 + k, k * c * fh * fw, -2, 2).reshape(k, c, fh, fw)
     ref = oracle_conv(x, f, dims)
     try:
-        b.use_test_library(True)
+        apply_config("auto", no_gather=1)
         for src in (b.SRC_NCHW, b.SRC_NCHW_FUSED):
             assert np.array_equal(gpu_conv(x, f, dims, mode, src_kind=src).astype(np.float64), ref), src
             assert b.last_kernel() == b.KERNEL_PERSISTENT
             nhwc = gpu_conv_nhwc(x, f, dims, mode, src)
             assert np.array_equal(np.transpose(nhwc, (0, 3, 1, 2)).astype(np.float64), ref), src
     finally:
-        b.use_test_library(False)
         reset_config()
 
 

@@ -1,0 +1,80 @@
+"""The gather kernel (conv_tc_gather.cu), forced, bit for bit against the oracle on small-integer data: filter tiles
+of every register layout, one to sixteen reduction slices, ragged reductions, unaligned filter rows, tiles that span
+images, and filter sizes without a specialisation."""
+import numpy as np
+import pytest
+
+from paper_2306_14320_b200 import binding as b
+from paper_2306_14320_b200 import workloads as wl
+from gpu_helpers import apply_config, ensure_built, gpu_conv, oracle_conv, reset_config
+from test_gpu_nhwc import gpu_conv_nhwc
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+# N, C, H, W, K, Fh, Fw, stride
+SHAPES = [
+    (1, 1, 1, 1, 1, 1, 1, 1), (1, 3, 32, 32, 16, 3, 3, 1), (2, 61, 19, 30, 32, 3, 4, 1), (3, 16, 21, 11, 160, 3, 4, 1),
+    (1, 256, 16, 16, 256, 3, 3, 1), (5, 7, 9, 9, 17, 3, 3, 1), (2, 33, 14, 13, 300, 1, 1, 2), (40, 5, 4, 3, 7, 2, 3, 1),
+    (1, 12, 33, 35, 70, 7, 7, 2), (1, 2, 51, 51, 24, 11, 11, 4), (2, 128, 10, 10, 130, 3, 3, 2), (1, 9, 20, 40, 33, 1, 7, 3),
+]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    ensure_built()
+
+
+@pytest.mark.parametrize("nt,z", [(0, 0), (16, 1), (32, 8), (64, 3), (128, 2), (256, 1), (192, 5), (16, 12), (48, 16)])
+@pytest.mark.parametrize("mode", [b.MODE_TF32, b.MODE_BF16], ids=["tf32", "bf16"])
+@pytest.mark.parametrize("dims", SHAPES, ids=lambda d: "x".join(map(str, d)))
+def test_gather_kernel_bit_exact(dims, mode, nt, z):
+    n, c, h, w, k, fh, fw, s = dims
+    stages = -(-c * fh * fw // 64)
+    if z > 1 and (z > stages or -(-stages // -(-stages // z)) != z):
+        pytest.skip("the reduction has no such cut")
+    x = wl.small_ints(41 + c, n * c * h * w).reshape(n, c, h, w)
+    f = wl.small_ints(42 + k, k * c * fh * fw, -2, 2).reshape(k, c, fh, fw)
+    ref = oracle_conv(x, f, dims)
+    try:
+        apply_config("generic", gather_nt=nt, gather_z=z)
+        for src in (b.SRC_NCHW, b.SRC_NCHW_FUSED):
+            assert np.array_equal(gpu_conv(x, f, dims, mode, src_kind=src).astype(np.float64), ref), src
+            assert b.last_kernel() == b.KERNEL_GATHER
+        xhat = np.stack([x[:, :, u:u + (ref.shape[2] - 1) * s + 1:s] for u in range(fh)], axis=-1)
+        xhat = np.ascontiguousarray(xhat.reshape(n, c, ref.shape[2], w * fh))
+        assert np.array_equal(gpu_conv(xhat, f, dims, mode, src_kind=b.SRC_IM2WIN).astype(np.float64), ref), "im2win"
+        nhwc = gpu_conv_nhwc(x, f, dims, mode, b.SRC_NCHW_FUSED)
+        assert np.array_equal(np.transpose(nhwc, (0, 3, 1, 2)).astype(np.float64), ref), "nhwc"
+    finally:
+        reset_config()
+
+
+@pytest.mark.parametrize("mode", [b.MODE_TF32, b.MODE_BF16], ids=["tf32", "bf16"])
+@pytest.mark.parametrize("dims", SHAPES, ids=lambda d: "x".join(map(str, d)))
+def test_gather_kernel_with_64_bit_indices_bit_exact(dims, mode):
+    """The form that tensors of 2^31 elements and more take, on small ones."""
+    n, c, h, w, k, fh, fw, s = dims
+    x = wl.small_ints(43 + c, n * c * h * w).reshape(n, c, h, w)
+    f = wl.small_ints(44 + k, k * c * fh * fw, -2, 2).reshape(k, c, fh, fw)
+    try:
+        apply_config("generic", gather_big=1)
+        assert np.array_equal(gpu_conv(x, f, dims, mode).astype(np.float64), oracle_conv(x, f, dims))
+    finally:
+        reset_config()
+
+
+def test_under_filled_layers_take_the_gather_kernel_and_large_ones_do_not():
+    try:
+        b.use_test_library(True)
+        for dims, want in (((1, 256, 16, 16, 256, 3, 3, 1), True), ((2, 20, 12, 13, 24, 3, 4, 1), True),
+                           ((32, 64, 58, 58, 64, 3, 3, 1), False)):
+            n, c, h, w, k, fh, fw, s = dims
+            x = wl.small_ints(5, n * c * h * w).reshape(n, c, h, w)
+            f = wl.small_ints(6, k * c * fh * fw, -2, 2).reshape(k, c, fh, fw)
+            for src in (b.SRC_NCHW, b.SRC_NCHW_FUSED):
+                gpu_conv(x, f, dims, b.MODE_BF16, src_kind=src)
+                assert (b.last_kernel() == b.KERNEL_GATHER) == want, (dims, src)
+    finally:
+        b.use_test_library(False)
+        reset_config()
