@@ -737,12 +737,14 @@ int choose_plan(const Geometry& g, Plan* best) {
 // kernel's three win) and the stride is 1 (with two column classes its T stages leave the rings too
 // little shared memory).  The persistent kernel's tiles may span images, this kernel's do not, so the
 // comparison is between the two kernels' waves: small images whose tiles just fill one wave there stay
-// there.  In BF16 mode a filter small enough to stay resident in the persistent kernel's shared memory
+// there.  In BF16 mode, and in TF32 mode fused, a filter small enough to stay resident in the persistent kernel's shared memory
 // also stays there.  Launches that fill less than half the SMs stay there too (reduction slices).
 template <int FH, int FW, int S, bool BF16, int SRCK>
 bool strip_preferred(const Geometry& g, const SParams& P) {
   if (S != 1 || P.NT < 96) return false;
   if (BF16 && (int64_t)g.K * g.Kg * 2 <= 160 * 1024) return false;
+  // (TF32 fused too: 128 images of 32x112x112, 96 filters, persistent 199 us, this kernel 288)
+  if (!BF16 && SRCK == 1 && P.n_ntiles == 1 && (int64_t)g.K * g.Kg * 4 <= 150 * 1024) return false;
   const int nsm = sm_count();
   const int64_t slots = P.pair ? nsm / 2 : nsm;
   const double strip_passes = (double)((P.units + slots - 1) / slots) * P.MH;

@@ -16,8 +16,12 @@
 // Sources: the fp32 or bf16 im2win tensor (entry u = 0 of strip h supplies (h, k); the last Fh-1 input
 // rows of a tile come from entries u > 0 of its last strip, so every byte of the tensor is fetched once
 // and nothing outside the tile's own strips is touched), or the untransformed input (the fused kind).
-// The filter operand is a tap-major copy F9[(u,v)][j][r] that a small kernel writes into the caller's
-// scratch at the start of the call, streamed by TMA boxes with the 64-byte swizzle.
+// The filter operand is a copy that a small kernel writes into the caller's scratch at the start of the call: the
+// filter stages one after the other, each the exact image of its shared memory (64-byte-swizzled rows), so that a
+// stage is one contiguous bulk copy.  (Boxes of 64-byte rows from a tap-major copy kept the copy engine busy for the
+// whole kernel: its rate of rows, not L2, fed the MMAs.  B200: 32 images of 384x15x15, 384 filters, TF32 from the
+// tensor 69 -> 62 us, fused 51 -> 46.5; 128 of 512x9x9, 512 filters, BF16 fused 77 -> 69.)  CTA pairs, whose copies signal the other CTA's barrier,
+// stream TMA boxes from a tap-major copy F9[(u,v)][j][r].
 //
 // Roles (one persistent CTA per SM, units t, t+grid, ...; a unit = 128*MH positions x one filter tile):
 //   warp 0       source producer (2-D TMA boxes, or one bulk copy per channel)
@@ -45,6 +49,7 @@ constexpr int kXMax = 3;  // X rows per interleaver thread and stage
 
 struct WParams {
   const void* src;
+  const uint8_t* fimg;  // single CTAs: the filter stages' images
   float* out;
   int32_t* status;
   int32_t C, K, Ho, Wo, W, H;
@@ -383,6 +388,8 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
         if (!wunit_at<PAIR>(P, it, rank, u)) break;
         if (P.bres && it > 0) break;  // resident filter: one unit's stages are the whole (single) filter tile
         const int32_t row0 = u.nt * P.NT + (int32_t)rank * P.NTB;
+        const uint8_t* fsrc = P.fimg + (size_t)u.nt * (size_t)(P.NXS * (FH * FW / P.TPS)) * P.b_stage_bytes;  // (a unit takes its tile's stages in order)
+        (void)row0; (void)fsrc;
         for (int32_t xs = 0; xs < P.NXS && ok; ++xs) {
           for (int32_t t0 = 0; t0 < FH * FW && ok; t0 += P.TPS, ++count, br.advance(P.SB)) {
             if (!P.bres) {
@@ -395,6 +402,10 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
 #endif
             if (!remote) ptx::mbar_arrive_expect_tx(full, P.b_stage_bytes * kShare);
             uint32_t dst = b_sa + (uint32_t)br.idx * P.b_stage_bytes;
+            if constexpr (!PAIR) {
+              ptx::bulk_g2s(dst, fsrc, P.b_stage_bytes, full);
+              fsrc += P.b_stage_bytes;
+            } else
             for (int32_t dt = 0; dt < P.TPS; ++dt)
               for (int32_t blk = 0; blk < nblk; ++blk, dst += (uint32_t)P.NTB * 64u) {
                 if (remote) tma_load_2d_pair(dst, &fmap, xs * P.G + blk * bke, (t0 + dt) * P.Kp + row0, full);
@@ -639,6 +650,50 @@ __global__ void __launch_bounds__(128) filter_tap_rows_kernel(const float* __res
   }
 }
 
+// The stages' images for single CTAs: stage (filter tile, channel group xs, TPS taps) = for each tap and each block of
+// 64 bytes of channels NT rows of 64 bytes, 16-byte chunk c of row r at chunk position c ^ ((r >> 1) & 3).
+template <bool BF16>
+__global__ void __launch_bounds__(128) filter_image_kernel(const float* __restrict__ f, uint8_t* __restrict__ o, int32_t K, int32_t NT,
+                                                           int32_t C, int32_t taps, int32_t TPS, int32_t G) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int ES = BF16 ? 2 : 4;
+  constexpr int BKE = 64 / ES;  // channels per row
+  __shared__ float sm[kPrepCh * kPrepTaps];
+  const int32_t j = (int32_t)blockIdx.x, tid = (int32_t)threadIdx.x;
+  const int32_t c0 = (int32_t)blockIdx.y * kPrepCh;
+  const int32_t nc = min(kPrepCh, C - c0);
+  const float* fj = f + ((int64_t)j * C + c0) * taps;
+  const int32_t n = nc * taps;
+  if (j < K) {
+    float v[kPrepTaps];
+#pragma unroll
+    for (int q = 0; q < kPrepTaps; ++q) {  // (all loads in flight before the first use)
+      const int32_t i = tid + q * 128;
+      v[q] = (q < taps && i < n) ? __ldg(fj + i) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < kPrepTaps; ++q) {
+      const int32_t i = tid + q * 128;
+      if (q < taps && i < n) sm[i] = v[q];
+    }
+  } else {
+    for (int32_t i = tid; i < n; i += 128) sm[i] = 0.f;
+  }
+  __syncthreads();
+  if (tid < nc) {
+    const int32_t nt = j / NT, r = j - nt * NT, ch = c0 + tid;
+    const int32_t xs = ch / G, blk = (ch - xs * G) / BKE, cb = (ch % BKE) * ES, nblk = G / BKE, nst = taps / TPS;
+    const size_t blk_bytes = (size_t)NT * 64, tap_bytes = blk_bytes * nblk;
+    uint8_t* d = o + ((size_t)(nt * (C / G) + xs) * nst * TPS) * tap_bytes + blk * blk_bytes +
+                 (size_t)((r >> 3) * 512 + (r & 7) * 64 + (((cb >> 4) ^ ((r >> 1) & 3)) << 4) + (cb & 15));
+    for (int32_t t = 0; t < taps; ++t, d += tap_bytes) {
+      const float x = sm[tid * taps + t];
+      if constexpr (BF16) *reinterpret_cast<__nv_bfloat16*>(d) = __float2bfloat16_rn(x);
+      else *reinterpret_cast<float*>(d) = x;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------------------- host side
 
 struct WPlan {
@@ -822,38 +877,42 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
 }
 
 // Which variant a problem gets (knobs override).  CTA pairs (each CTA fetches half the filter rows) where they
-// were measured faster than single CTAs: the 5x5 layers in BF16 mode with 256-wide filter tiles (25 taps make
-// the filter stream the largest consumer of shared-memory bandwidth), with one block per tile so that two
-// accumulator buffers remain; and 192-wide tiles in TF32 mode from the fused source and in BF16 mode from the
-// bf16 tensor.  Elsewhere a pair's MMAs, which cost the issuing thread about twice as long, lose more than the
-// halved filter traffic gains.
+// were measured faster than single CTAs with their contiguous filter stages: the 5x5 layers in BF16 mode with 256-wide
+// filter tiles (with one block per tile, so that two accumulator buffers remain: 27x27 outputs 129 and 133 us) and in
+// TF32 mode fused with more than 64 filters (64 images of 64x40x40, 128 filters, 71 and 79 us; 256 filters 141 and 148);
+// and the TF32 fused 3x3 layers of 65 to 128 filters on long rows, whose 256-row tiles leave the rings of a single CTA
+// too little (112x112 439 and 473 us, 61x61 133 and 137; 56x56 123 and 122).  Elsewhere a pair's MMAs, which cost the
+// issuing thread about twice as long, lose more than the halved filter traffic gains.
 // Rows per tile: the number of 128-row blocks that gives the least estimated time: rounds of units over the
-// SMs (or pairs) x (blocks per unit + the fixed part of a unit, measured as about two blocks); ties go to the
-// taller tile.
+// SMs (or pairs) x (blocks per unit + the fixed part of a unit, below); ties go to the taller tile.
 template <int FH, int FW, bool BF16, int SRCK>
 int choose_wplan(const Geometry& g, WPlan* best) {
   const int forced = knobs().window_mh & 255;
   const int nt = (((g.K + (g.K + 255) / 256 - 1) / ((g.K + 255) / 256)) + 15) / 16 * 16;
   int pair = 0;
-  if (FH == 5) pair = BF16 && nt >= 192 && (int64_t)g.Ho * g.W >= 640;  // (faster on the 27x27-output 5x5 layer, slower on the 20x20 one)
-  else if (nt >= 192 && nt < 256) pair = (SRCK == 1 && !BF16) || SRCK == 2;
+  if (FH == 5) pair = BF16 ? nt >= 256 && (int64_t)g.Ho * g.W >= 640 : SRCK == 1 && nt > 64;  // (BF16: slower on 20x20 outputs)
+  else if (SRCK == 1 && !BF16) pair = nt > 64 && nt <= 128 && g.W >= 60;
   if (knobs().window_pair == 1) pair = 1;
   if (knobs().window_pair == 2) pair = 0;
   for (int attempt = 0; attempt < 2; ++attempt, pair = 1 - pair) {
     if (attempt == 1 && knobs().window_pair) break;  // (a forced variant that does not fit: unsupported)
-    int64_t best_cost = -1;
+    double best_cost = -1;
+    // a unit's time beside its blocks, in blocks: the halo rows of X and the tile's hand-overs weigh more the fewer
+    // filters share them (measured: 31x31 images, 160 filters, TF32 fused, one block 101 us, two 114; 58x58, 64 filters,
+    // BF16 fused, 27 and 21)
+    const double fixed = nt <= 64 ? 2.0 : (nt < 128 ? 1.0 : 0.25);
     WPlan cand;
     const int64_t slots = pair ? sm_count() / 2 : sm_count();
     for (int mh = 2; mh >= 1; mh /= 2) {  // (four blocks per tile were measured too: never faster, and they leave the rings less room)
       if (forced && mh != forced) continue;
-      if (!forced && pair && FH == 5 && mh != 1) continue;
+      if (!forced && pair && FH == 5 && BF16 && mh != 1) continue;
       if (make_wplan<FH, FW, BF16, SRCK>(g, &cand, pair, mh) != IM2WIN_OK) continue;
       if (!forced && mh > 1 && (int64_t)g.Ho * g.W <= 128 * (mh / 2)) continue;  // the image fits fewer blocks
       // tiles of up to 128 filters keep two accumulator buffers (the epilogue overlaps the next unit); wider
       // ones gain more from the second block (each filter stage feeds two MMAs)
       if (!forced && cand.P.NT <= 128 && cand.P.ND < 2) continue;
       const int64_t rounds = (cand.P.units + slots - 1) / slots;
-      const int64_t cost = rounds * (mh + 2);  // (a unit costs about two blocks' time beside its blocks: measured)
+      const double cost = (double)rounds * (mh + fixed);
       if (best_cost < 0 || cost < best_cost) { best_cost = cost; *best = cand; }
     }
     if (best_cost >= 0) return IM2WIN_OK;
@@ -866,7 +925,10 @@ int choose_wplan(const Geometry& g, WPlan* best) {
 // both modes).  Its strengths: the staged bytes and the interleaving work are a third of the strip-matrix
 // kernel's, and it has no per-thread window loads (the persistent kernel's bound on deep layers in BF16 mode).
 // In TF32 mode and for the fused source the 256-wide filter tiles on images of more than one block stay with
-// the strip-matrix kernel's CTA pairs; TF32 layers of 64 filters from the fp32 im2win tensor stay with the
+// the strip-matrix kernel's CTA pairs, and those of 65 to 128 filters come here from 64 channels on (64 images of
+// 96x58x58, 128 filters: 87 us, strip-matrix 107, persistent 124; 32 channels, 96 filters on 112x112: 236, persistent 199);
+// 5x5 layers fused come here in both modes (TF32: 128 images of 32x30x30, 64 filters, 40 us, persistent 55; 64 of
+// 64x40x40, 128 filters, 71 and 119); TF32 layers of 64 filters from the fp32 im2win tensor stay with the
 // persistent kernel (a 64-column MMA from shared memory takes 54 cycles, that kernel's from tensor memory 32,
 // and the tensor's staged bytes are three times the input's), the same layers fused come here; and where the
 // persistent kernel finishes in a single wave of tiles that span images (small images, one filter tile) that
@@ -875,11 +937,11 @@ template <int FH, int FW, bool BF16, int SRCK>
 bool window_preferred(const Geometry& g, const WParams& P) {
   const int nsm = sm_count();
   if (P.units * 2 <= nsm) return false;  // under-filled launches: the persistent kernel's reduction slices
-  if (FH == 5) return BF16 || (SRCK == 0 && P.RPI < 640);  // 5x5 layers: 25 taps of one staged tile (TF32: from the tensor, smaller images)
+  if (FH == 5) return BF16 || SRCK == 1 || P.RPI < 640;  // 5x5 layers: 25 taps of one staged tile (TF32: from the tensor, smaller images)
   const int64_t span_tiles = (g.Mtot + 127) / 128;
   if (P.n_ntiles == 1 && span_tiles <= nsm && P.NT > 128) return false;  // one wave of the persistent kernel
   if (!BF16) {
-    if (SRCK == 1) return P.NT <= 64 || (g.C >= 128 && P.NT >= 128 && P.NT <= 192);
+    if (SRCK == 1) return P.NT <= 64 || (g.C >= 64 && P.NT <= 128) || (g.C >= 128 && P.NT <= 192);
     return P.NT > 64 && P.NT <= 192;
   }
   if (SRCK == 2) return P.NT <= 192 || P.RPI >= 128;                   // bf16 im2win tensor
@@ -942,6 +1004,7 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   EncodeTiledFn enc = encode_fn();
   if (!enc) return IM2WIN_EUNSUPPORTED;
   P.src = src; P.out = out;
+  P.fimg = static_cast<const uint8_t*>(scratch.ptr);
 #ifdef IM2WIN_PROF
   P.prof = g_prof;
   P.skip = knobs().window_mh >> 8;   // (profiling build: ablation bits ride in the upper bits of the tile-height switch)
@@ -952,7 +1015,7 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   CUtensorMap fmap, xmap;
   memset(&fmap, 0, sizeof(fmap));
   memset(&xmap, 0, sizeof(xmap));
-  {
+  if (P.pair) {
     const cuuint64_t gdim[2] = {(cuuint64_t)g.C, (cuuint64_t)FH * FW * P.Kp};
     const cuuint64_t gstr[1] = {(cuuint64_t)g.C * (BF16 ? 2 : 4)};
     const cuuint32_t box[2] = {(cuuint32_t)(BF16 ? 32 : 16), (cuuint32_t)P.NTB};
@@ -978,8 +1041,8 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
     }
   }
   const dim3 pgrid((unsigned)P.Kp, (unsigned)((g.C + kPrepCh - 1) / kPrepCh));
-  if (BF16) filter_tap_rows_kernel<true><<<pgrid, 128, 0, st>>>(f, scratch.ptr, g.K, P.Kp, g.C, FH * FW);
-  else filter_tap_rows_kernel<false><<<pgrid, 128, 0, st>>>(f, scratch.ptr, g.K, P.Kp, g.C, FH * FW);
+  if (P.pair) filter_tap_rows_kernel<BF16><<<pgrid, 128, 0, st>>>(f, scratch.ptr, g.K, P.Kp, g.C, FH * FW);
+  else filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, g.C, FH * FW, P.TPS, P.G);
   if (cudaGetLastError() != cudaSuccess) return IM2WIN_ECUDA;
   rc = P.pair ? launch_wkernel<FH, FW, BF16, SRCK, true>(P, pl, fmap, xmap, st) : launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
   if (rc != IM2WIN_OK) return rc;
