@@ -299,6 +299,13 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
                                  /*fused=*/from_input, /*behind_transform=*/from_input);
   };
   rc = general_first ? take_general() : IM2WIN_EUNSUPPORTED;
+  // The window-offset kernel stages a third (3x3) or a fifth (5x5) of the bytes from the input, which SRC_NCHW has at
+  // hand beside the im2win tensor.  (B200: 32 images of 384x15x15, 384 filters, TF32 62 us from the tensor, 47 from the
+  // input; 128 of 160x31x31, 160 filters, TF32 120 and 101.)  Not below about 2e9 multiplications, where its filter copy is
+  // a third launch that counts (27 images of 32x37x37, 32 filters, BF16: 20 us a call, 16 with the persistent kernel).
+  if (rc == IM2WIN_EUNSUPPORTED && general && src_kind == IM2WIN_SRC_NCHW && !knobs().force_generic &&
+      (double)g.n_out * (double)g.Kg >= 2e9)
+    rc = launch_conv_tc_window(src, filter, out_nchw, g, mode, st, scratch, 1, out16);
   if (rc == IM2WIN_EUNSUPPORTED && !knobs().force_generic) rc = launch_conv_tc(xhat, filter, out_nchw, g, mode, st, scratch, 0, out16);
   if (rc == IM2WIN_EUNSUPPORTED && general && !general_first) rc = take_general();
   return rc;
