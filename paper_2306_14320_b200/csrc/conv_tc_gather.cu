@@ -486,7 +486,13 @@ bool gather_preferred(const Geometry& g, int mode, bool fused) {
   if (k.no_strip || k.force_strip || k.no_window || k.force_window || k.no_box || k.no_pim || k.bslice || k.no_gather) return false;
   if (g.Mtot > 128 * 300) return false;
   const bool bf16 = mode == IM2WIN_MODE_BF16;
-  return gather_plan(g, bf16, fused, 256).us < 0.8 * persistent_us(g, bf16);
+  const double limit = 0.8 * persistent_us(g, bf16);
+  // (no cut takes less than this: most calls are decided without looking at the cuts, 2 us of host time)
+  const int64_t tiles = (g.Mtot + 127) / 128, stages = (g.Kg + kBK - 1) / kBK;
+  int64_t z = tiles < sm_count() ? sm_count() / tiles : 1;
+  if (z > kGMaxZ) z = kGMaxZ;
+  if (5.0 + (double)((stages + z - 1) / z) * (bf16 ? 0.8 : 1.2) >= limit) return false;
+  return gather_plan(g, bf16, fused, 256).us < limit;
 }
 
 int launch_conv_tc_gather(const float* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
