@@ -309,7 +309,8 @@ struct TileParams {
   int32_t* status;
   int32_t H, W, s, Ho, L;
   int32_t MB, nblk, PB;
-  int32_t QW;           // column quads per row: ceil(W / 4)
+  int32_t QW;           // transposition units per row: column quads, ceil(W / 4), or (cols) single columns, W
+  int32_t cols;
   int64_t planes, HW, HoL, n_in_total;
   uint64_t magic_QW;    // ceil(2^32 / QW)
   uint64_t magic_MQ;    // ceil(2^32 / (rows per plane in the job * QW))
@@ -317,6 +318,51 @@ struct TileParams {
   uint32_t off_out;     // byte offset of the output buffer in shared memory
   uint32_t off_bar;     // byte offset of the mbarrier
 };
+
+__device__ __forceinline__ float lds_f32(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts_f32(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void sts_u16(uint32_t a, uint16_t v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory"); }
+
+// The transposition where rows have an odd length (and FH is odd): every strip starts at another 16-byte phase, so quads
+// of columns would read and write element by element, four lanes to a bank.  A thread takes one column instead:
+// neighbouring lanes read neighbouring floats and write FH floats apart, both without bank conflicts.
+// tin_a, tout_a: shared addresses of the range's first element; a column outside the ranges is recorded, not copied.
+// (B200, batch 128: 11x11 stride 4 on 227x227 62.6 -> 53.4 us, 5.4 TB/s; 7x7 stride 2 on 225x225 70.7 -> 58.5; 3x3 on
+// 512 channels of 9x9 19.2 -> 16.5, of 256 channels of 15x15 24.7 -> 22.2.)
+template <int FH, bool OUT16>
+__device__ __forceinline__ void transpose_columns(const TileParams& P, uint32_t tin_a, uint32_t tout_a, int32_t npl, int32_t mb,
+                                                  int32_t n_in, int32_t n_out, int32_t plane_floats, int32_t out_plane) {
+  constexpr uint32_t OS = OUT16 ? 2u : 4u;
+  const int32_t W = P.W, sW = P.s * W, units_plane = mb * W, nunits = npl * units_plane;
+  const int32_t in_last = n_in - (FH - 1) * W - 1, out_last = n_out - FH;
+  for (int32_t q = threadIdx.x; q < nunits; q += kThreads) {
+    int32_t pl = 0, rem = q;
+    if (npl > 1) {
+      pl = (int32_t)(((uint64_t)(uint32_t)q * P.magic_MQ) >> 32);
+      rem = q - pl * units_plane;
+    }
+    const int32_t mm = (int32_t)(((uint64_t)(uint32_t)rem * P.magic_QW) >> 32);
+    const int32_t k = rem - mm * W;
+    const int32_t si = pl * plane_floats + mm * sW + k, oi = pl * out_plane + mm * P.L + k * FH;
+    if (si < 0 || si > in_last || oi < 0 || oi > out_last) {
+      atomicCAS(P.status, 0, (int32_t)DEV_RANGE);
+      continue;
+    }
+    const uint32_t src = tin_a + (uint32_t)si * 4u, dst = tout_a + (uint32_t)oi * OS;
+    float r[FH];
+#pragma unroll
+    for (int u = 0; u < FH; ++u) r[u] = lds_f32(src + (uint32_t)(u * W) * 4u);
+#pragma unroll
+    for (int u = 0; u < FH; ++u) {
+      if constexpr (OUT16) sts_u16(dst + (uint32_t)u * OS, bf16_rn(r[u]));
+      else sts_f32(dst + (uint32_t)u * OS, r[u]);
+    }
+  }
+}
 
 // OUT16: the output is the bf16 storage variant (P.out then points at 16-bit words).
 template <int FH, bool OUT16>
@@ -393,7 +439,10 @@ __global__ void __launch_bounds__(kThreads) transform_tile_kernel(const TilePara
   OutT* const tout = tout0 + dskew;                               // tout[e] <-> out[dst0 + e]
   const int32_t sW = P.s * P.W;
   const int32_t units_plane = mb * P.QW;
-  const int32_t nunits = npl * units_plane;
+  const int32_t nunits = P.cols ? 0 : npl * units_plane;
+  if (P.cols)
+    transpose_columns<FH, OUT16>(P, ptx::smem_u32(tin0) + (uint32_t)skew * 4u, ptx::smem_u32(tout0) + (uint32_t)dskew * (uint32_t)sizeof(OutT),
+                                 npl, mb, n_in, n_out, plane_floats, out_plane);
   const bool in_even = ((P.W | skew) & 1) == 0;                  // every row start is 8-byte aligned
   for (int32_t q = threadIdx.x; q < nunits; q += kThreads) {
     int32_t pl = 0, rem = q;
@@ -522,6 +571,11 @@ int launch_transform_tile(const float* in, void* out, bool out16, const Geometry
   // small planes (several whole planes per CTA): 28 KB, eight CTAs per SM, measured 3-8 % faster on the
   // launch- and tail-bound layers; row blocks of larger planes keep 34 KB (shorter blocks re-read more rows)
   if (hw + g.HoL <= 7168 - 16) kBudget = 7168 - 16;
+  // odd rows (transposed column by column, see the kernel) under tall filters: 48 KB, four CTAs per SM; their output rows
+  // are so long that 34 KB hold two (11x11 on 227x227: 62 us with two per CTA, 53 with three, 58 with four)
+  const bool odd_rows = (g.W & 1) && (g.Fh & 1) && g.Fh > 1;
+  const bool tall = odd_rows && g.Fh >= 7 && hw + g.HoL > 7168 - 16;
+  if (tall) kBudget = 12288 - 16;
   if (knobs().transform_budget_kb) kBudget = (int64_t)knobs().transform_budget_kb * 256 - 16;  // (test build)
   int32_t PB = 1, MB = g.Ho, nblk = 1;
   if (hw + g.HoL <= kBudget) {
@@ -538,7 +592,9 @@ int launch_transform_tile(const float* in, void* out, bool out16, const Geometry
     // neighbouring blocks re-read Fh - s rows each; with the output buffer taking most of the
     // budget, wide rows leave blocks so short that this would dominate: leave those to the
     // staged-gather kernel, which stages the input only
-    if ((int64_t)(g.Fh - g.s) * 8 > (int64_t)(MB - 1) * g.s + g.Fh) return IM2WIN_EUNSUPPORTED;
+    // (column by column: a sixth of the CTA's traffic, most of which is output)
+    if (tall ? (int64_t)(g.Fh - g.s) * 6 > (int64_t)MB * (g.s + g.Fh) : (int64_t)(g.Fh - g.s) * 8 > (int64_t)(MB - 1) * g.s + g.Fh)
+      return IM2WIN_EUNSUPPORTED;
   }
   const int64_t ctas = nblk == 1 ? (planes + PB - 1) / PB : planes * nblk;
   if (ctas > INT32_MAX) return IM2WIN_EUNSUPPORTED;
@@ -551,7 +607,10 @@ int launch_transform_tile(const float* in, void* out, bool out16, const Geometry
   if (!P.status) return IM2WIN_ECUDA;
   P.H = g.H; P.W = g.W; P.s = g.s; P.Ho = g.Ho; P.L = g.L;
   P.MB = MB; P.nblk = nblk; P.PB = PB;
-  P.QW = (g.W + 3) / 4;
+  const int64_t rows_out = nblk == 1 ? g.Ho : MB;
+  // (five rows and a CTA per plane: quads are 0-3 % faster, 31x31 36.9 and 38.0 us)
+  P.cols = odd_rows && !(g.Fh == 5 && PB == 1) && rows_out * g.W * PB * rows_out * g.W < ((int64_t)1 << 32);
+  P.QW = P.cols ? g.W : (g.W + 3) / 4;
   {
     // honoured for single-CTA problems only: every CTA would wait out its own second otherwise
     P.test_skip_copy = (knobs().test_skip_copy && ctas == 1) ? 1 : 0;
