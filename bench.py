@@ -41,8 +41,8 @@ NOMINAL_TF32_OVER_BF16 = 1.1 / 2.25
 NCU_TRAFFIC_BYTES = {("resnet3x3", "tf32"): 319.52e6 + 83.52e6, ("stem7x7", "tf32"): 277.09e6 + 352.88e6,
                      ("down3x3", "tf32"): 322.35e6 + 74.64e6,
                      ("deep3x3", "tf32"): 90.54e6 + 4.44e6, ("deep3x3", "bf16"): 89.36e6 + 3.78e6}
-KERNEL_NAMES = {1: "conv_tc_strip_kernel", 2: "conv_tc_persistent_kernel", 3: "conv_tc_kernel", 4: "conv_fp32_kernel",
-                5: "conv_tc_window_kernel"}
+KERNEL_NAMES = {1: "conv_tc_strip_kernel", 2: "conv_tc_persistent_kernel", 4: "conv_fp32_kernel",
+                5: "conv_tc_window_kernel", 6: "conv_tc_gather_kernel"}
 
 
 def _peaks():
@@ -128,10 +128,12 @@ def kernel_used(layer, mode_name, torch, b):
     try:
         b.use_test_library(True)
         ws = torch.zeros(b.conv_workspace_bytes(dims, b.SRC_NCHW, mode) // 4 + 64, dtype=torch.float32, device="cuda")
+        off = (b.workspace_bytes(dims) + 255) // 256 * 256 // 4
         x = torch.zeros((layer.N, layer.C, layer.H, layer.W), dtype=torch.float32, device="cuda")
         f = torch.zeros((layer.K, layer.C, layer.Fh, layer.Fw), dtype=torch.float32, device="cuda")
         out = torch.empty((layer.N, layer.K, ho, wo), dtype=torch.float32, device="cuda")
-        b.conv(x, b.SRC_NCHW, f, dims, mode, out, ws)
+        b.transform(x, dims, ws)  # (the step's two calls: the convolution reads the im2win tensor)
+        b.conv(ws, b.SRC_IM2WIN, f, dims, mode, out, ws[off:])
         torch.cuda.synchronize()
         return KERNEL_NAMES.get(b.last_kernel(), "unknown")
     except (ImportError, OSError, RuntimeError, AttributeError):

@@ -111,7 +111,8 @@ int im2win_transform_bf16(const float* in_nchw, const im2win_shape* shape, uint1
  * (Algorithm 2 prints the strip offset as n*s*Wf+v*Hf+u, which equals the above for Hf==Wf and
  * is the form consistent with Algorithm 1 otherwise.)
  * src:       device.  src_kind NCHW: the input I (N*C*H*W floats); the call first runs the
- *            transform into `workspace`, which then holds Ihat and may be reused by the caller.
+ *            transform into `workspace`, which then holds Ihat and may be reused by the caller (the
+ *            convolution reads Ihat or, where that is faster, the input itself: the same values).
  *            src_kind IM2WIN: an im2win tensor; `workspace` may be NULL, or give scratch (see below).
  *            src_kind NCHW_FUSED: the input I; the tensor-core kernel stages the input rows a tile
  *            needs and reads the windows from them, so nothing of size Ihat is written (workspace
