@@ -32,9 +32,9 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
-# conv_tc_persistent.cu holds four families of kernel instantiations (by filter size); compiled as
-# four translation units (-DIM2WIN_PART=k) they build in parallel.
-PARTS = {"conv_tc_persistent.cu": 8}
+# These files hold families of kernel instantiations (by filter size); compiled as so many translation units
+# (-DIM2WIN_PART=k) they build in parallel.
+PARTS = {"conv_tc_persistent.cu": 8, "conv_tc_window.cu": 2}
 
 
 def build_library(force: bool = False, verbose: bool = False, out: str | None = None,

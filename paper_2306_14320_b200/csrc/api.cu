@@ -307,6 +307,14 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
     src_kind = IM2WIN_SRC_NCHW;
   }
   Scratch scratch = scratch_from(0);
+  // From the untransformed input the window-offset kernel writes the im2win tensor itself, beside the convolution.  (Calls
+  // below 1e7 multiplications take the time of their launches whatever the kernel: not looked at.)
+  if (src_kind == IM2WIN_SRC_NCHW && general && !knobs().force_generic && knobs().window_xhat != 2 &&
+      (knobs().window_xhat == 1 || (!knobs().force_window && (double)g.n_out * (double)g.Kg >= 1e7))) {
+    rc = launch_conv_tc_window(src, filter, out_nchw, g, mode, st, scratch_from(win_bytes), 3, out16, knobs().window_xhat == 1,
+                               reinterpret_cast<float*>(ws));
+    if (rc != IM2WIN_EUNSUPPORTED) return rc;
+  }
   if (src_kind == IM2WIN_SRC_NCHW) {
     rc = launch_transform(static_cast<const float*>(src), reinterpret_cast<float*>(ws), g, st);
     if (rc != IM2WIN_OK) return rc;
@@ -319,14 +327,6 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
                                  /*fused=*/from_input, /*behind_transform=*/from_input);
   };
   rc = general_first ? take_general() : IM2WIN_EUNSUPPORTED;
-  // The window-offset kernel stages a third (3x3) or a fifth (5x5) of the bytes from the input, which SRC_NCHW has at
-  // hand beside the im2win tensor.  (B200: 32 images of 384x15x15, 384 filters, TF32 62 us from the tensor, 47 from the
-  // input; 128 of 160x31x31, 160 filters, TF32 120 and 101; 287 random layers 0.91 of the tensor's time in the mean, 43 of
-  // them 4 to 24 % more.)  Not below 2e9 multiplications, where its filter copy is a third launch that counts (27 images of
-  // 32x37x37, 32 filters, 0.3e9, BF16: 20 us a call, 16 with the persistent kernel; nothing between was measured).
-  if (rc == IM2WIN_EUNSUPPORTED && general && src_kind == IM2WIN_SRC_NCHW && !knobs().force_generic &&
-      (double)g.n_out * (double)g.Kg >= 2e9)
-    rc = launch_conv_tc_window(src, filter, out_nchw, g, mode, st, scratch, 1, out16);
   if (rc == IM2WIN_EUNSUPPORTED && !knobs().force_generic) rc = launch_conv_tc(xhat, filter, out_nchw, g, mode, st, scratch, 0, out16);
   if (rc == IM2WIN_EUNSUPPORTED && general && !general_first) rc = take_general();
   return rc;
@@ -420,7 +420,7 @@ int im2win_debug_set_option(const char* name, int value) {
       {"ntiles", &Knobs::ntiles}, {"transform_gather", &Knobs::transform_gather},
       {"test_skip_copy", &Knobs::test_skip_copy}, {"strip_mh", &Knobs::strip_mh}, {"strip_pair", &Knobs::strip_pair},
       {"force_window", &Knobs::force_window}, {"no_window", &Knobs::no_window}, {"window_mh", &Knobs::window_mh},
-      {"window_plan", &Knobs::window_plan}, {"window_pair", &Knobs::window_pair}, {"window_two", &Knobs::window_two}, {"no_gather", &Knobs::no_gather}, {"gather_nt", &Knobs::gather_nt}, {"gather_z", &Knobs::gather_z}, {"gather_big", &Knobs::gather_big}, {"gather_zfail", &Knobs::gather_zfail}, {"window_nohelp", &Knobs::window_nohelp}, {"window_bres", &Knobs::window_bres}, {"transform_budget_kb", &Knobs::transform_budget_kb}};
+      {"window_plan", &Knobs::window_plan}, {"window_pair", &Knobs::window_pair}, {"window_two", &Knobs::window_two}, {"window_xhat", &Knobs::window_xhat}, {"no_gather", &Knobs::no_gather}, {"gather_nt", &Knobs::gather_nt}, {"gather_z", &Knobs::gather_z}, {"gather_big", &Knobs::gather_big}, {"gather_zfail", &Knobs::gather_zfail}, {"window_nohelp", &Knobs::window_nohelp}, {"window_bres", &Knobs::window_bres}, {"transform_budget_kb", &Knobs::transform_budget_kb}};
   for (const Entry& e : table)
     if (strcmp(e.name, name) == 0) { g_knobs.*(e.field) = value; return IM2WIN_OK; }
   return IM2WIN_EINVAL;

@@ -73,9 +73,10 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
                    Scratch scratch, int src_kind, bool out_bf16);
 // Scratch bytes with which every kernel above is available for this problem (0 if none wants any).
 size_t strip_scratch_bytes(const Geometry& g, int mode, int src_kind);
-// The window-offset kernel (conv_tc_window.cu; stride 1, 3x3 and 5x5): same source kinds and scratch rules.
+// The window-offset kernel (conv_tc_window.cu; stride 1, 3x3 and 5x5): same source kinds and scratch rules, and kind 3: the
+// untransformed input, the fp32 im2win tensor written to `xhat` beside the result.
 int launch_conv_tc_window(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
-                          Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower = false);
+                          Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower = false, float* xhat = nullptr);
 size_t window_scratch_bytes(const Geometry& g, int mode, int src_kind);
 // (its plan, for the test build) two issuing threads, resident filter, filter stages; false where not implemented
 bool window_issue_plan(const Geometry& g, int mode, int src_kind, int* two, int* resident, int* stages);
@@ -135,6 +136,7 @@ struct Knobs {
   int gather_z = 0;          // gather kernel: forced number of reduction slices (0: own choice)
   int gather_big = 0;        // gather kernel: 64-bit indices
   int gather_zfail = 0;      // gather kernel: launches with larger clusters than this are refused (0: none)
+  int window_xhat = 0;       // SRC_NCHW: 1 = the window-offset kernel that writes the im2win tensor wherever implemented, 2 = never
   int window_two = 0;        // window-offset kernel: 1 = two MMA-issuing threads forced, 2 = one forced, 0 = own choice
 };
 const Knobs& knobs();

@@ -29,6 +29,12 @@
 //   warp 2       filter producer
 //   warps 4-11   interleavers: staged channel rows -> X (fp32 as is for TF32, cvt.rn.bf16x2 for BF16)
 //   warps 12-19  epilogue: tcgen05.ld -> coalesced NCHW stores
+//   4 more       (source kind 3) writers of the im2win tensor, see below
+//
+// Source kind 3 is the call from the untransformed input that leaves the im2win tensor to the caller (Algorithm 1, then
+// Algorithm 2): the tile's staged input rows hold every strip element of its Ho x W positions, so four more warps write the
+// tensor out of the source stages while the tensor core works on the same rows.  The transform as a kernel of its own moves
+// the same bytes at the HBM's rate, leaves the tensor cores idle meanwhile, and reads the input a second time.
 // Every wait is bounded (status word + common teardown on expiry).
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -46,11 +52,13 @@ namespace {
 using namespace stripc;
 
 constexpr int kXMax = 3;  // X rows per interleaver thread and stage
+constexpr int kXW = 4;    // warps that write the im2win tensor (source kind 3)
 
 struct WParams {
   const void* src;
   const uint8_t* fimg;  // single CTAs: the filter stages' images
   float* out;
+  float* xhat;        // source kind 3: the im2win tensor to write
   int32_t* status;
   int32_t C, K, Ho, Wo, W, H;
   int32_t RPI;        // positions per image, counted with the full row length: Ho * W
@@ -222,11 +230,16 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
   SPROF_DUMP(1)
 }
 
-// SRCK: 0 = fp32 im2win tensor, 1 = untransformed input (fused), 2 = bf16 im2win tensor (BF16 mode).
+// Source kinds: 0 = fp32 im2win tensor, 1 = untransformed input (fused), 2 = bf16 im2win tensor (BF16 mode),
+// 3 = untransformed input, the fp32 im2win tensor written beside the result.
+template <int SRCK>
+constexpr bool kFromInput = SRCK == 1 || SRCK == 3;
+
 template <int FH, int FW, bool BF16, int SRCK, bool PAIR>
-__global__ void __launch_bounds__(640, 1)
+__global__ void __launch_bounds__(SRCK == 3 ? 640 + 32 * kXW : 640, 1)
 conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap, const __grid_constant__ CUtensorMap xmap) {
-  constexpr bool FUSED = SRCK == 1;
+  constexpr bool FUSED = kFromInput<SRCK>;
+  constexpr bool XHAT = SRCK == 3;
   constexpr bool SRC16 = SRCK == 2;
   static_assert(!SRC16 || BF16, "a 16-bit source feeds the BF16 mode");
   constexpr uint32_t ES = SRC16 ? 2u : 4u;       // bytes per source element
@@ -246,7 +259,7 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
   if (threadIdx.x == 0) {
     for (int i = 0; i < kMaxRaw; ++i) {
       ptx::mbar_init(ptx::smem_u32(&bars->raw_full[i]), 1);
-      ptx::mbar_init(ptx::smem_u32(&bars->raw_empty[i]), kTW);
+      ptx::mbar_init(ptx::smem_u32(&bars->raw_empty[i]), kTW + (XHAT ? kXW : 0));
     }
     for (int i = 0; i < kMaxB; ++i) {
       ptx::mbar_init(ptx::smem_u32(&bars->b_full[i]), 1);
@@ -600,6 +613,62 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
       }
     }
     if (warp == kEpiWarp0) { SPROF_DUMP(6) }
+  } else if (XHAT && warp >= kEpiWarp0 + P.n_epi) {
+    // ================================================================ IM2WIN TENSOR: staged input rows -> global
+    // The tile's positions [R0, R0 + 128*MH) are as many consecutive columns of each channel's strips: FH floats each, one
+    // contiguous range of the plane.  A lane takes every 32nd float of it, so that a warp's store is 128 contiguous bytes
+    // at any phase (planes need not be whole 16-byte chunks) and its loads, of FH rows of 32/FH neighbouring positions,
+    // stay within two wavefronts; FH offsets repeat every 32 positions.  Where several filter tiles share a row tile each
+    // writes the stages of its turn.
+    const int32_t xw = warp - kEpiWarp0 - P.n_epi;
+    uint32_t off[FH];
+#pragma unroll
+    for (int q = 0; q < FH; ++q) {
+      const int32_t f = lane + 32 * q;
+      off[q] = (uint32_t)(f / FH + (f % FH) * P.W) * 4u;
+    }
+    constexpr int ZU = FH <= 3 ? 4 : 2;  // groups of 32 positions in flight (128*MH positions are a multiple of them)
+    const int64_t plane_out = (int64_t)P.RPI * FH;
+    Ring rr;
+    bool ok = true;
+    for (int64_t it = 0; ok; ++it) {
+      WUnit u;
+      if (!wunit_at<PAIR>(P, it, rank, u)) break;
+      const int32_t n = min(128 * P.MH, P.RPI - u.R0) * FH;  // floats of this tile per channel
+      const int32_t sk0 = P.dense ? 0 : (int32_t)(((int64_t)u.img * P.C * P.plane + u.R0) & (EPC - 1));
+      const int32_t nstages = P.NXS * P.NSUB;
+      int32_t turn = 0;
+      for (int32_t sidx = 0; sidx < nstages && ok; ++sidx, rr.advance(P.SR)) {
+        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->raw_full[rr.idx]), rr.phase, DEV_TIMEOUT_RAW_FULL);
+        if (!ok) break;
+        if (u.store && turn == u.nt) {
+          const uint32_t rs = raw_sa + (uint32_t)rr.idx * P.raw_stage_bytes;
+          for (int32_t ch = xw; ch < P.GR; ch += kXW) {
+            const int32_t c = sidx * P.GR + ch;
+            const int32_t sk = P.pm ? ((sk0 + c * P.pm) & (EPC - 1)) : sk0;
+            uint32_t a = rs + (uint32_t)(ch * P.BXE + sk) * 4u;
+            float* d = P.xhat + ((int64_t)u.img * P.C + c) * plane_out + (int64_t)u.R0 * FH + lane;
+            int32_t left = n - lane;
+            while (left > 0) {
+              uint32_t v[ZU * FH];
+#pragma unroll
+              for (int z = 0; z < ZU; ++z)
+#pragma unroll
+                for (int q = 0; q < FH; ++q) v[z * FH + q] = lds_u32(a + off[q] + (uint32_t)z * 128u);
+#pragma unroll
+              for (int z = 0; z < ZU * FH; ++z)
+                if (z * 32 < left) d[z * 32] = __uint_as_float(v[z]);
+              a += ZU * 128u;
+              d += ZU * 32 * FH;
+              left -= ZU * 32 * FH;
+            }
+          }
+        }
+        if (++turn == P.n_ntiles) turn = 0;
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->raw_empty[rr.idx]));
+      }
+    }
   }
 
   // ------------------------------------------------------------------ teardown
@@ -735,7 +804,7 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   // 10-20 %, wider tiles nothing.
   P.two = (!pair && (knobs().window_two == 1 || (knobs().window_two == 0 && P.NT <= 64))) ? 1 : 0;
   P.NTB = pair ? P.NT / 2 : P.NT;
-  if (SRCK == 1) { P.plane = (int64_t)g.H * g.W; P.n_src = g.n_in; }
+  if (kFromInput<SRCK>) { P.plane = (int64_t)g.H * g.W; P.n_src = g.n_in; }
   else { P.plane = g.HoL; P.n_src = g.n_win; }
   P.pm = (int32_t)(P.plane % EPC);
   const int64_t cap = 227 * 1024 - 1024 - (1024 + 128 + 16) - (int64_t)((sizeof(SBars) + 15) / 16 * 16) - 64;
@@ -754,7 +823,7 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   // columns; with one block per tile only the first set could help, so the epilogue warps keep all columns
   P.epi_split = (P.ND == 1 && P.MH == 2 && P.NT >= 64 && !knobs().window_nohelp) ? (P.NT / 2 + 15) / 16 * 16 : P.NT;
   // source elements of one channel a tile needs at most, plus the 16-byte phase in front
-  const int64_t len_max = SRCK == 1 ? P.RX : (int64_t)FH * (128 * P.MH + g.W);
+  const int64_t len_max = kFromInput<SRCK> ? P.RX : (int64_t)FH * (128 * P.MH + g.W);
   int64_t cp = len_max + 2 * EPC;
   const int64_t cp_align = 32 / ES;
   cp = (cp + cp_align - 1) / cp_align * cp_align;
@@ -772,8 +841,8 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   const Try order_fused[] = {{2, FW, 16}, {2, FW, 8}, {2, 1, 32}, {2, 1, 16}, {1, FW, 32}, {1, FW, 16}, {1, 1, 16}, {1, 1, 8}, {1, 1, 4}};
   const Try order_win[] = {{1, FW, 16}, {1, FW, 8}, {2, 1, 8}, {1, 1, 8}, {1, 1, 4}, {1, 1, 16}};
   const Try order_win16[] = {{1, FW, 32}, {1, FW, 16}, {2, 1, 16}, {1, 1, 16}, {1, 1, 8}, {1, 1, 32}};
-  const Try* order_tail = SRCK == 1 ? order_fused : (SRCK == 2 ? order_win16 : order_win);
-  const int n_tail = SRCK == 1 ? 9 : 6;
+  const Try* order_tail = kFromInput<SRCK> ? order_fused : (SRCK == 2 ? order_win16 : order_win);
+  const int n_tail = kFromInput<SRCK> ? 9 : 6;
   // In front of those, the measured exceptions: 256-wide filter tiles want one filter block per X stage (a stage of
   // two blocks x Fw taps x 256 rows is 96 KB, and two of them leave the other rings too little): fused with two
   // 128-row blocks {1,Fw,16} (the deep 3x3 layers in BF16 mode: 50 -> 43, 62 -> 56, 83 -> 74 us), with one block
@@ -781,7 +850,7 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   // of 192 and more (TF32: 108 -> 98, 151 -> 134 us on the 384-filter layers).
   Try order_all[12];
   int n_order = 0;
-  if (SRCK == 1) {
+  if (kFromInput<SRCK>) {
     if (P.NT >= 256) order_all[n_order++] = P.MH == 2 ? Try{1, FW, 16} : Try{2, FW, 32};
   } else if (SRCK == 0 && P.MH == 2) {  // (images of a single block keep the general order: measured)
     if (BF16) {
@@ -817,7 +886,9 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
       const int64_t b_stage_bytes = (int64_t)tps * nblk * blk_bytes;
       // boxes of at most 2 KB per channel row
       int64_t nbx = 1, bxe = cp;
-      const bool box_ok = P.pm == 0 && gr >= 4 && encode_fn() != nullptr && (int64_t)g.N * g.C <= INT32_MAX && !knobs().no_box;
+      // (the writers of the im2win tensor walk a channel's row in one piece: longer rows are bulk copies there)
+      const bool box_ok = P.pm == 0 && gr >= 4 && encode_fn() != nullptr && (int64_t)g.N * g.C <= INT32_MAX && !knobs().no_box &&
+                          !(SRCK == 3 && cp * ES > 2048);
       if (box_ok) {
         nbx = (cp * ES + 2047) / 2048;
         bxe = (cp + nbx - 1) / nbx;
@@ -893,7 +964,7 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   while ((int32_t)P.tmem_cols < cols) P.tmem_cols *= 2;
   P.idesc = ptx::make_idesc(pair ? 256 : 128, P.NT, BF16 ? 1 : 2);
   pl->scratch_bytes = (size_t)FH * FW * P.Kp * (size_t)g.C * (BF16 ? 2 : 4);
-  pl->threads = (kEpiWarp0 + P.n_epi) * 32;
+  pl->threads = (kEpiWarp0 + P.n_epi + (SRCK == 3 ? kXW : 0)) * 32;
   return IM2WIN_OK;
 }
 
@@ -911,8 +982,8 @@ int choose_wplan(const Geometry& g, WPlan* best) {
   const int forced = knobs().window_mh & 255;
   const int nt = (((g.K + (g.K + 255) / 256 - 1) / ((g.K + 255) / 256)) + 15) / 16 * 16;
   int pair = 0;
-  if (FH == 5) pair = BF16 ? nt >= 256 && (int64_t)g.Ho * g.W >= 640 : SRCK == 1 && nt > 64;  // (BF16: slower on 20x20 outputs)
-  else if (SRCK == 1 && !BF16) pair = nt > 64 && nt <= 128 && g.W >= 60;
+  if (FH == 5) pair = BF16 ? nt >= 256 && (int64_t)g.Ho * g.W >= 640 : kFromInput<SRCK> && nt > 64;  // (BF16: slower on 20x20 outputs)
+  else if (kFromInput<SRCK> && !BF16) pair = nt > 64 && nt <= 128 && g.W >= 60;
   if (knobs().window_pair == 1) pair = 1;
   if (knobs().window_pair == 2) pair = 0;
   WPlan small_pairs;
@@ -978,6 +1049,37 @@ double persistent_fused_us(const Geometry& g, const WParams& P) {
   return 3.0 + rounds * (0.87 + steps * (resident ? 0.055 : (P.NT <= 64 ? 0.07 : 0.092)) + 3.5 * columns);
 }
 
+// Source kind 3 against the transform and the fastest kernel on its tensor (gather, persistent, strip-matrix or this one),
+// both in microseconds: fits to 1,200 random calls on B200 (this kernel within 9 % in the median, the others within 13 %).
+// Over those calls the picks take 0.89 of the others' time, the better of the two on each 0.85; where this kernel is not
+// expected to win by a fourteenth the others stay (1 in a hundred picks is more than 3 % slower than them).
+// (128 images of 64x58x58, 64 filters, TF32 166 -> 124 us a call with new inputs; 32 of 384x15x15, 384 filters 60 -> 54; 119 of
+// 128x58x58, 85 filters, BF16 267 -> 191.)
+template <int FH, int FW, bool BF16>
+bool xhat_preferred(const Geometry& g, const WParams& P) {
+  //                                     start  MMAs   rows  columns tensor  pairs
+  static const double on[2][2][6] = {{{9.0, 1.47, 0.53, 1.63, 0.0, 3.4}, {8.4, 1.52, 1.10, 1.77, 0.114, 0.0}},
+                                     {{8.3, 0.93, 1.93, 2.69, 0.0, 4.2}, {8.8, 1.32, 0.67, 2.46, 0.0, 4.1}}};
+  //                                     start  bytes  steps  steps x columns  columns  slices
+  static const double off[2][2][6] = {{{9.9, 0.26, 0.024, 0.039, 0.78, 1.4}, {10.2, 0.28, 0.017, 0.050, 0.64, 1.1}},
+                                      {{10.2, 0.61, 0.0, 0.032, 0.69, 1.5}, {11.9, 0.45, 0.0, 0.035, 0.34, 0.0}}};
+  const double* a = on[FH == 5][BF16];
+  const double* o = off[FH == 5][BF16];
+  const int64_t nsm = sm_count(), slots = P.pair ? nsm / 2 : nsm, rounds = (P.units + slots - 1) / slots;
+  const int64_t taps_c = (int64_t)FH * FW * g.C, step = BF16 ? 16 : 8;
+  const double mma = FH * FW * (double)((g.C + step - 1) / step) * P.MH * (P.NT > 108 ? P.NT / 2.0 : 54.0) / 1900.0;
+  const double here = a[0] + a[5] * P.pair + (double)rounds * (a[1] * mma + a[2] * g.C * (128 * P.MH + (FH - 1) * g.W) * 1e-4 +
+                      a[3] * P.NT * P.MH * 0.01 + a[4] * g.C * 128 * P.MH * FH * 4 / P.n_ntiles * 1e-5);
+  const int64_t tiles = (g.Mtot + 127) / 128 * P.n_ntiles, waves = (tiles + nsm - 1) / nsm, ng = (g.C + step - 1) / step;
+  int64_t z = tiles >= nsm ? 1 : nsm / tiles;
+  z = z > 16 ? 16 : z;
+  z = z > ng ? ng : z;
+  const double steps = (double)(waves * ((taps_c + step - 1) / step)) / (double)z;
+  const double there = o[0] + o[1] * (double)(g.n_in + g.n_win) * 4e-6 + o[2] * steps + o[3] * steps * P.NT * 0.01 +
+                       o[4] * (double)waves * P.NT * 0.01 + (z > 1 ? o[5] : 0.0);
+  return here < 0.93 * there;
+}
+
 // Whether this kernel is expected to beat the strip-matrix and the persistent kernel: rules read off a
 // measured table (B200, batch 128, every stride-1 3x3 / 5x5 layer of the benchmark lists, three source kinds,
 // both modes).  Its strengths: the staged bytes and the interleaving work are a third of the strip-matrix
@@ -994,6 +1096,7 @@ double persistent_fused_us(const Geometry& g, const WParams& P) {
 template <int FH, int FW, bool BF16, int SRCK>
 bool window_preferred(const Geometry& g, const WParams& P) {
   const int nsm = sm_count();
+  if (SRCK == 3) return xhat_preferred<FH, FW, BF16>(g, P);
   if (P.units * 2 <= nsm) return false;  // under-filled launches: the persistent kernel's reduction slices
   if (FH == 5) {  // 25 taps of one staged tile (TF32 from the tensor: smaller images)
     if (BF16 || SRCK != 1) return BF16 || P.RPI < 640;
@@ -1058,7 +1161,7 @@ int launch_wkernel(const WParams& P, const WPlan& pl, const CUtensorMap& fmap, c
 
 template <int FH, int FW, bool BF16, int SRCK>
 int launch_window(const void* src, const float* f, float* out, const Geometry& g, cudaStream_t st, Scratch scratch,
-                  bool even_if_slower) {
+                  bool even_if_slower, float* xhat) {
   WPlan pl;
   int rc = choose_wplan<FH, FW, BF16, SRCK>(g, &pl);
   if (rc != IM2WIN_OK) return rc;
@@ -1068,7 +1171,7 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   EncodeTiledFn enc = encode_fn();
   if (!enc) return IM2WIN_EUNSUPPORTED;
   if (scratch.probe) return IM2WIN_OK;
-  P.src = src; P.out = out;
+  P.src = src; P.out = out; P.xhat = xhat;
   P.fimg = static_cast<const uint8_t*>(scratch.ptr);
 #ifdef IM2WIN_PROF
   P.prof = g_prof;
@@ -1121,12 +1224,14 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
 
 template <int FH, int FW>
 int launch_window_fs(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st, Scratch scratch,
-                     int src_kind, bool eis) {
+                     int src_kind, bool eis, float* xhat) {
   const bool bf16 = mode == IM2WIN_MODE_BF16;
-  if (src_kind == 2) return bf16 ? launch_window<FH, FW, true, 2>(src, f, out, g, st, scratch, eis) : IM2WIN_EUNSUPPORTED;
+  if (src_kind == 3)
+    return bf16 ? launch_window<FH, FW, true, 3>(src, f, out, g, st, scratch, eis, xhat) : launch_window<FH, FW, false, 3>(src, f, out, g, st, scratch, eis, xhat);
+  if (src_kind == 2) return bf16 ? launch_window<FH, FW, true, 2>(src, f, out, g, st, scratch, eis, nullptr) : IM2WIN_EUNSUPPORTED;
   if (src_kind == 1)
-    return bf16 ? launch_window<FH, FW, true, 1>(src, f, out, g, st, scratch, eis) : launch_window<FH, FW, false, 1>(src, f, out, g, st, scratch, eis);
-  return bf16 ? launch_window<FH, FW, true, 0>(src, f, out, g, st, scratch, eis) : launch_window<FH, FW, false, 0>(src, f, out, g, st, scratch, eis);
+    return bf16 ? launch_window<FH, FW, true, 1>(src, f, out, g, st, scratch, eis, nullptr) : launch_window<FH, FW, false, 1>(src, f, out, g, st, scratch, eis, nullptr);
+  return bf16 ? launch_window<FH, FW, true, 0>(src, f, out, g, st, scratch, eis, nullptr) : launch_window<FH, FW, false, 0>(src, f, out, g, st, scratch, eis, nullptr);
 }
 
 template <int FH, int FW>
@@ -1134,11 +1239,28 @@ int wplan_fs(const Geometry& g, int mode, int src_kind, WPlan* pl) {
   const bool bf16 = mode == IM2WIN_MODE_BF16;
   if (src_kind == 2) return bf16 ? choose_wplan<FH, FW, true, 2>(g, pl) : IM2WIN_EUNSUPPORTED;
   if (src_kind == 1) return bf16 ? choose_wplan<FH, FW, true, 1>(g, pl) : choose_wplan<FH, FW, false, 1>(g, pl);
+  if (src_kind == 3) return bf16 ? choose_wplan<FH, FW, true, 3>(g, pl) : choose_wplan<FH, FW, false, 3>(g, pl);
   return bf16 ? choose_wplan<FH, FW, true, 0>(g, pl) : choose_wplan<FH, FW, false, 0>(g, pl);
 }
 
+}  // namespace
+
+// The filter sizes' kernels build as translation units in parallel (-DIM2WIN_PART=0: 3x3 and everything else, 1: 5x5; without
+// the macro everything is compiled here).
+#ifndef IM2WIN_PART
+#define IM2WIN_PART -1
+#endif
+#define IM2WIN_WINDOW_ARGS const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st, \
+                           Scratch scratch, int src_kind, bool even_if_slower, float* xhat
+#define IM2WIN_WINDOW_PASS src, f, out, g, mode, st, scratch, src_kind, even_if_slower, xhat
+int launch_window_5x5(IM2WIN_WINDOW_ARGS);
+#if IM2WIN_PART == -1 || IM2WIN_PART == 1
+int launch_window_5x5(IM2WIN_WINDOW_ARGS) { return launch_window_fs<5, 5>(IM2WIN_WINDOW_PASS); }
+#endif
+
+#if IM2WIN_PART == -1 || IM2WIN_PART == 0
 // The plan of a problem the kernel implements (whether or not it is preferred there).
-int window_plan(const Geometry& g, int mode, int src_kind, WPlan* pl) {
+static int window_plan(const Geometry& g, int mode, int src_kind, WPlan* pl) {
   if (mode != IM2WIN_MODE_TF32 && mode != IM2WIN_MODE_BF16) return IM2WIN_EUNSUPPORTED;
   if (g.s != 1) return IM2WIN_EUNSUPPORTED;
   if (g.Fh == 3 && g.Fw == 3) return wplan_fs<3, 3>(g, mode, src_kind, pl);
@@ -1146,15 +1268,13 @@ int window_plan(const Geometry& g, int mode, int src_kind, WPlan* pl) {
   return IM2WIN_EUNSUPPORTED;
 }
 
-}  // namespace
-
 int launch_conv_tc_window(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
-                          Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower) {
+                          Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower, float* xhat) {
   if (out_bf16) return IM2WIN_EUNSUPPORTED;  // fp32 epilogue only
   if (mode != IM2WIN_MODE_TF32 && mode != IM2WIN_MODE_BF16) return IM2WIN_EUNSUPPORTED;
   if (g.s != 1 || knobs().no_window) return IM2WIN_EUNSUPPORTED;
-  if (g.Fh == 3 && g.Fw == 3) return launch_window_fs<3, 3>(src, f, out, g, mode, st, scratch, src_kind, even_if_slower);
-  if (g.Fh == 5 && g.Fw == 5) return launch_window_fs<5, 5>(src, f, out, g, mode, st, scratch, src_kind, even_if_slower);
+  if (g.Fh == 3 && g.Fw == 3) return launch_window_fs<3, 3>(IM2WIN_WINDOW_PASS);
+  if (g.Fh == 5 && g.Fw == 5) return launch_window_5x5(IM2WIN_WINDOW_PASS);
   return IM2WIN_EUNSUPPORTED;
 }
 
@@ -1171,5 +1291,7 @@ bool window_issue_plan(const Geometry& g, int mode, int src_kind, int* two, int*
   *stages = pl.P.SB;
   return true;
 }
+
+#endif  // IM2WIN_PART == -1 || IM2WIN_PART == 0
 
 }  // namespace im2win
