@@ -20,8 +20,10 @@
 // filter stages one after the other, each the exact image of its shared memory (64-byte-swizzled rows), so that a
 // stage is one contiguous bulk copy.  (Boxes of 64-byte rows from a tap-major copy kept the copy engine busy for the
 // whole kernel: its rate of rows, not L2, fed the MMAs.  B200: 32 images of 384x15x15, 384 filters, TF32 from the
-// tensor 69 -> 62 us, fused 51 -> 46.5; 128 of 512x9x9, 512 filters, BF16 fused 77 -> 69.)  CTA pairs, whose copies signal the other CTA's barrier,
-// stream TMA boxes from a tap-major copy F9[(u,v)][j][r].
+// tensor 69 -> 62 us, fused 51 -> 46.5; 128 of 512x9x9, 512 filters, BF16 fused 77 -> 69.)  CTA pairs, whose copies signal the
+// leader's barrier, which an untiled bulk copy cannot, fetch their half of a stage's image as one box of 1 KB rows.  (With
+// boxes of 64-byte rows the MMA thread waited 94 of 217 kcycles for filter stages, now 35 of 163: 128 images of 96x31x31, 256
+// 5x5 filters, BF16 from the bf16 tensor, convolution 128 -> 109 us.)
 //
 // Roles (one persistent CTA per SM, units t, t+grid, ...; a unit = 128*MH positions x one filter tile):
 //   warp 0       source producer (2-D TMA boxes, or one bulk copy per channel)
@@ -56,7 +58,7 @@ constexpr int kXW = 4;    // warps that write the im2win tensor (source kind 3)
 
 struct WParams {
   const void* src;
-  const uint8_t* fimg;  // single CTAs: the filter stages' images
+  const uint8_t* fimg;  // the filter stages' images
   float* out;
   float* xhat;        // source kind 3: the im2win tensor to write
   int32_t* status;
@@ -395,8 +397,6 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
       int64_t count = 0;
       bool ok = true;
       SPROF_DECL
-      const int32_t bke = BF16 ? 32 : 16;  // elements (channels) per 64-byte filter row
-      const int32_t nblk = P.G / bke;
       asm volatile("griddepcontrol.wait;" ::: "memory");  // the filter copy is written by the kernel launched just before
       // Pair mode: this CTA fetches its half of every block's rows, and the bytes of both CTAs are counted on
       // the leader's barrier: the leader announces both halves with its one arrival, the other CTA only
@@ -407,9 +407,12 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
         WUnit u;
         if (!wunit_at<PAIR>(P, it, rank, u)) break;
         if (P.bres && it > 0) break;  // resident filter: one unit's stages are the whole (single) filter tile
-        const int32_t row0 = u.nt * P.NT + (int32_t)rank * P.NTB;
-        const uint8_t* fsrc = P.fimg + (size_t)u.nt * (size_t)(P.NXS * (FH * FW / P.TPS)) * P.b_stage_bytes;  // (a unit takes its tile's stages in order)
-        (void)row0; (void)fsrc;
+        // (a unit takes its tile's stages in order; of each a pair's CTAs take a half)
+        const int32_t stage0 = u.nt * P.NXS * (FH * FW / P.TPS);
+        const uint8_t* fsrc = P.fimg + (size_t)stage0 * P.b_stage_bytes;
+        const int32_t rows = (int32_t)(P.b_stage_bytes >> 10);  // (pairs) 1 KB rows of a half
+        int32_t row = (stage0 * 2 + (int32_t)rank) * rows;
+        (void)fsrc; (void)row;
         for (int32_t xs = 0; xs < P.NXS && ok; ++xs) {
           for (int32_t t0 = 0; t0 < FH * FW && ok; t0 += P.TPS, ++count, br.advance(P.SB)) {
             if (!P.bres) {
@@ -421,16 +424,15 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
             if (P.skip & 2) { if (!remote) ptx::mbar_arrive(full); continue; }
 #endif
             if (!remote) ptx::mbar_arrive_expect_tx(full, P.b_stage_bytes * kShare);
-            uint32_t dst = b_sa + (uint32_t)br.idx * P.b_stage_bytes;
+            const uint32_t dst = b_sa + (uint32_t)br.idx * P.b_stage_bytes;
             if constexpr (!PAIR) {
               ptx::bulk_g2s(dst, fsrc, P.b_stage_bytes, full);
               fsrc += P.b_stage_bytes;
-            } else
-            for (int32_t dt = 0; dt < P.TPS; ++dt)
-              for (int32_t blk = 0; blk < nblk; ++blk, dst += (uint32_t)P.NTB * 64u) {
-                if (remote) tma_load_2d_pair(dst, &fmap, xs * P.G + blk * bke, (t0 + dt) * P.Kp + row0, full);
-                else tma_load_2d(dst, &fmap, xs * P.G + blk * bke, (t0 + dt) * P.Kp + row0, full);
-              }
+            } else {
+              if (remote) tma_load_2d_pair(dst, &fmap, 0, row, full);
+              else tma_load_2d(dst, &fmap, 0, row, full);
+              row += 2 * rows;
+            }
           }
         }
       }
@@ -682,55 +684,15 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
   }
 }
 
-// Tap-major copy of the filter for the TMA-streamed B operand:
-//   F9[t][j][r] = F[j][r][u][v],  t = u*Fw + v   (j < K; rows K..Kp-1 are zero), fp32 or bf16 (nearest even).
-// One CTA per (filter j, block of 128 channels): its 128*Fh*Fw values pass through shared memory, so that both
-// the reads and the writes are contiguous, and every CTA is one load - store round trip (the convolution
-// kernel's first MMA waits for this copy: its latency counts).
 constexpr int kPrepCh = 128, kPrepTaps = 25;
-template <bool BF16>
-__global__ void __launch_bounds__(128) filter_tap_rows_kernel(const float* __restrict__ f, void* __restrict__ o, int32_t K,
-                                                              int32_t Kp, int32_t C, int32_t taps) {
-  // the convolution kernel that follows may start its prologue now (it waits for this grid's completion
-  // before it reads the copy)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  __shared__ float sm[kPrepCh * kPrepTaps];
-  const int32_t j = (int32_t)blockIdx.x, tid = (int32_t)threadIdx.x;
-  const int32_t c0 = (int32_t)blockIdx.y * kPrepCh;
-  const int32_t nc = min(kPrepCh, C - c0);
-  const float* fj = f + ((int64_t)j * C + c0) * taps;
-  const int32_t n = nc * taps;
-  if (j < K) {
-    float v[kPrepTaps];
-#pragma unroll
-    for (int q = 0; q < kPrepTaps; ++q) {  // (all loads in flight before the first use)
-      const int32_t i = tid + q * 128;
-      v[q] = (q < taps && i < n) ? __ldg(fj + i) : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < kPrepTaps; ++q) {
-      const int32_t i = tid + q * 128;
-      if (q < taps && i < n) sm[i] = v[q];
-    }
-  } else {
-    for (int32_t i = tid; i < n; i += 128) sm[i] = 0.f;
-  }
-  __syncthreads();
-  if (tid < nc) {
-    for (int32_t t = 0; t < taps; ++t) {
-      const float x = sm[tid * taps + t];
-      const int64_t oi = ((int64_t)t * Kp + j) * C + c0 + tid;
-      if (BF16) static_cast<__nv_bfloat16*>(o)[oi] = __float2bfloat16_rn(x);
-      else static_cast<float*>(o)[oi] = x;
-    }
-  }
-}
-
-// The stages' images for single CTAs: stage (filter tile, channel group xs, TPS taps) = for each tap and each block of
-// 64 bytes of channels NT rows of 64 bytes, 16-byte chunk c of row r at chunk position c ^ ((r >> 1) & 3).
+// The stages' images: stage (filter tile, channel group xs, TPS taps) = for each half of the filter tile (CTA pairs; else
+// the whole tile, NTB = NT) and each tap and each block of 64 bytes of channels NTB rows of 64 bytes, 16-byte chunk c of row
+// r at chunk position c ^ ((r >> 1) & 3).  One CTA per (filter j, block of 128 channels): its 128*Fh*Fw values pass through
+// shared memory, so that the reads are contiguous, and every CTA is one load - store round trip (the convolution kernel's
+// first MMA waits for this copy: its latency counts).
 template <bool BF16>
 __global__ void __launch_bounds__(128) filter_image_kernel(const float* __restrict__ f, uint8_t* __restrict__ o, int32_t K, int32_t NT,
-                                                           int32_t C, int32_t taps, int32_t TPS, int32_t G) {
+                                                           int32_t NTB, int32_t C, int32_t taps, int32_t TPS, int32_t G) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int ES = BF16 ? 2 : 4;
   constexpr int BKE = 64 / ES;  // channels per row
@@ -757,15 +719,17 @@ __global__ void __launch_bounds__(128) filter_image_kernel(const float* __restri
   }
   __syncthreads();
   if (tid < nc) {
-    const int32_t nt = j / NT, r = j - nt * NT, ch = c0 + tid;
+    const int32_t nt = j / NT, half = (j - nt * NT) / NTB, r = j - nt * NT - half * NTB, ch = c0 + tid, nhalf = NT / NTB;
     const int32_t xs = ch / G, blk = (ch - xs * G) / BKE, cb = (ch % BKE) * ES, nblk = G / BKE, nst = taps / TPS;
-    const size_t blk_bytes = (size_t)NT * 64, tap_bytes = blk_bytes * nblk;
-    uint8_t* d = o + ((size_t)(nt * (C / G) + xs) * nst * TPS) * tap_bytes + blk * blk_bytes +
+    const size_t blk_bytes = (size_t)NTB * 64, tap_bytes = blk_bytes * nblk, stage_bytes = tap_bytes * TPS;
+    uint8_t* d = o + ((size_t)(nt * (C / G) + xs) * nst * nhalf + half) * stage_bytes + blk * blk_bytes +
                  (size_t)((r >> 3) * 512 + (r & 7) * 64 + (((cb >> 4) ^ ((r >> 1) & 3)) << 4) + (cb & 15));
-    for (int32_t t = 0; t < taps; ++t, d += tap_bytes) {
+    const size_t skip = (size_t)(nhalf - 1) * stage_bytes;  // the other half's
+    for (int32_t t = 0, dt = 1; t < taps; ++t, ++dt, d += tap_bytes) {
       const float x = sm[tid * taps + t];
       if constexpr (BF16) *reinterpret_cast<__nv_bfloat16*>(d) = __float2bfloat16_rn(x);
       else *reinterpret_cast<float*>(d) = x;
+      if (dt == TPS) { dt = 0; d += skip; }
     }
   }
 }
@@ -1184,13 +1148,14 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   memset(&fmap, 0, sizeof(fmap));
   memset(&xmap, 0, sizeof(xmap));
   if (P.pair) {
-    const cuuint64_t gdim[2] = {(cuuint64_t)g.C, (cuuint64_t)FH * FW * P.Kp};
-    const cuuint64_t gstr[1] = {(cuuint64_t)g.C * (BF16 ? 2 : 4)};
-    const cuuint32_t box[2] = {(cuuint32_t)(BF16 ? 32 : 16), (cuuint32_t)P.NTB};
+    // the images as rows of 1 KB (128 8-byte elements): a half of a stage is a whole number of them, 16 filter rows each
+    const cuuint64_t gdim[2] = {128, (cuuint64_t)(pl.scratch_bytes >> 10)};
+    const cuuint64_t gstr[1] = {1024};
+    const cuuint32_t box[2] = {128, (cuuint32_t)(P.b_stage_bytes >> 10)};
     const cuuint32_t estr[2] = {1, 1};
-    if (enc(&fmap, BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, scratch.ptr, gdim, gstr, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    if (box[1] > 256 || gdim[1] > INT32_MAX ||
+        enc(&fmap, CU_TENSOR_MAP_DATA_TYPE_INT64, 2, scratch.ptr, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return IM2WIN_EUNSUPPORTED;
   }
   if (P.box) {
@@ -1209,8 +1174,7 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
     }
   }
   const dim3 pgrid((unsigned)P.Kp, (unsigned)((g.C + kPrepCh - 1) / kPrepCh));
-  if (P.pair) filter_tap_rows_kernel<BF16><<<pgrid, 128, 0, st>>>(f, scratch.ptr, g.K, P.Kp, g.C, FH * FW);
-  else filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, g.C, FH * FW, P.TPS, P.G);
+  filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, P.NTB, g.C, FH * FW, P.TPS, P.G);
   if (cudaGetLastError() != cudaSuccess) return IM2WIN_ECUDA;
   rc = P.pair ? launch_wkernel<FH, FW, BF16, SRCK, true>(P, pl, fmap, xmap, st) : launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
   if (rc != IM2WIN_OK) return rc;
