@@ -61,6 +61,12 @@ int make_geometry(const im2win_shape* sh, Geometry* g) {
   return IM2WIN_OK;
 }
 
+// (configurations of the test build that force or exclude a kernel choose among the others)
+static bool images_first() {
+  const Knobs& k = knobs();
+  return k.strip_images == 1 || !(k.no_strip || k.force_strip || k.force_window || k.no_window);
+}
+
 int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                    Scratch scratch, int src_kind, bool out_bf16) {
   // src_kind: 0 = fp32 im2win tensor, 1 = untransformed input consumed fused, 2 = bf16 im2win tensor.
@@ -68,6 +74,8 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
   // the persistent specialised kernel.  (Where none applies, the caller takes the general kernel.)
   int rc = IM2WIN_EUNSUPPORTED;
   if (!knobs().force_generic) {
+    if (images_first()) rc = launch_conv_tc_strip_images(src, f, out, g, mode, st, scratch, src_kind, out_bf16);
+    if (rc != IM2WIN_EUNSUPPORTED) return rc;
     rc = launch_conv_tc_window(src, f, out, g, mode, st, scratch, src_kind, out_bf16);
     if (rc != IM2WIN_EUNSUPPORTED) return rc;
     if (!knobs().no_strip) rc = launch_conv_tc_strip(src, f, out, g, mode, st, scratch, src_kind, out_bf16);
@@ -270,7 +278,8 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
   if (src_kind == IM2WIN_SRC_NCHW_FUSED) {
     auto specialised = [&](Scratch sc) {
       if (mode == IM2WIN_MODE_FP32 || knobs().force_generic) return (int)IM2WIN_EUNSUPPORTED;
-      int r = launch_conv_tc_window(xhat, filter, out_nchw, g, mode, st, sc, 1, out16);
+      int r = images_first() ? launch_conv_tc_strip_images(xhat, filter, out_nchw, g, mode, st, sc, 1, out16) : (int)IM2WIN_EUNSUPPORTED;
+      if (r == IM2WIN_EUNSUPPORTED) r = launch_conv_tc_window(xhat, filter, out_nchw, g, mode, st, sc, 1, out16);
       if (r == IM2WIN_EUNSUPPORTED && !knobs().no_strip) r = launch_conv_tc_strip(xhat, filter, out_nchw, g, mode, st, sc, 1, out16);
       if (r == IM2WIN_EUNSUPPORTED)
         r = launch_conv_tc_persistent(xhat, filter, out_nchw, g, mode, st, sc, /*fused=*/true, /*src_bf16=*/false, out16);
@@ -418,7 +427,7 @@ int im2win_debug_set_option(const char* name, int value) {
       {"no_bslice", &Knobs::no_bslice}, {"splitk", &Knobs::splitk}, {"force_stream", &Knobs::force_stream},
       {"nsets", &Knobs::nsets}, {"no_l2ahead", &Knobs::no_l2ahead}, {"no_btma", &Knobs::no_btma},
       {"ntiles", &Knobs::ntiles}, {"transform_gather", &Knobs::transform_gather},
-      {"test_skip_copy", &Knobs::test_skip_copy}, {"strip_mh", &Knobs::strip_mh}, {"strip_pair", &Knobs::strip_pair},
+      {"test_skip_copy", &Knobs::test_skip_copy}, {"strip_mh", &Knobs::strip_mh}, {"strip_images", &Knobs::strip_images}, {"strip_pair", &Knobs::strip_pair},
       {"force_window", &Knobs::force_window}, {"no_window", &Knobs::no_window}, {"window_mh", &Knobs::window_mh},
       {"window_plan", &Knobs::window_plan}, {"window_pair", &Knobs::window_pair}, {"window_two", &Knobs::window_two}, {"window_xhat", &Knobs::window_xhat}, {"no_gather", &Knobs::no_gather}, {"gather_nt", &Knobs::gather_nt}, {"gather_z", &Knobs::gather_z}, {"gather_big", &Knobs::gather_big}, {"gather_zfail", &Knobs::gather_zfail}, {"window_nohelp", &Knobs::window_nohelp}, {"window_bres", &Knobs::window_bres}, {"transform_budget_kb", &Knobs::transform_budget_kb}};
   for (const Entry& e : table)

@@ -66,6 +66,9 @@ struct Scratch {
 // be the fastest -- for sources no other kernel accepts)
 int launch_conv_tc_strip(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                          Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower = false);
+// Several whole small images per tile of the strip-matrix kernel, where that is the fastest way.
+int launch_conv_tc_strip_images(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
+                                Scratch scratch, int src_kind, bool out_bf16);
 int launch_conv_tc_persistent(const void* src, const float* f, float* out, const Geometry& g, int mode,
                               cudaStream_t st, Scratch scratch, bool fused = false, bool src_bf16 = false,
                               bool out_bf16 = false);
@@ -122,6 +125,7 @@ struct Knobs {
   int transform_budget_kb = 0;  // transform tile kernel: shared-memory budget per CTA in KB (0: own choice)
   int transform_gather = 0;  // transform: the staged-gather kernel instead of the tile kernel
   int test_skip_copy = 0;    // transform tile kernel, single-CTA problems: announce the input copy, never issue it
+  int strip_images = 0;      // strip-matrix kernel, several images per tile: 1 = in forced configurations too, 2 = never, 0 = own choice
   int strip_mh = 0;          // strip-matrix kernel: 128-row halves per tile (0: own choice)
   int strip_pair = 0;        // strip-matrix kernel: 1 = CTA pairs (cta_group::2) forced, 2 = single CTAs forced, 0 = own choice
   int force_window = 0;      // use the window-offset kernel (conv_tc_window.cu) wherever it is implemented

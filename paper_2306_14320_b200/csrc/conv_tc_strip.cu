@@ -14,8 +14,8 @@
 // (Stride s > 1: the columns are split into s classes k mod s, one T matrix per class; tap v reads class
 // v mod s at row offset v / s.)
 //
-// GEMM view per work unit: M = 128*MH consecutive rows p = m*WP + q of one image (WP = ceil(W/s); the
-// rows with q >= Wo are computed and dropped), N = a tile of up to 256 filters, K = (r,u) per tap.
+// GEMM view per work unit: M = 128*MH consecutive rows p = m*WP + q of one image, or of several whole small images
+// (WP = ceil(W/s); the rows with q >= Wo are computed and dropped), N = a tile of up to 256 filters, K = (r,u) per tap.
 // Roles (one persistent CTA per SM, units t, t+grid, ...):
 //   warp 0       source producer: one 2-D TMA box (or one bulk copy per channel) per group of GR channels
 //   warp 1       MMA issuer (one thread): tcgen05.mma kind::tf32 / kind::f16, A and B from shared memory,
@@ -49,6 +49,8 @@ struct SParams {
   int32_t C, K, Ho, Wo, W, WP;
   int32_t RPI;        // T rows per image: Ho * WP
   int32_t TPI;        // tiles per image
+  int32_t IPT;        // whole images per tile (1: a tile lies in one image); N images in all
+  int32_t N;
   int32_t MH;         // 128-row halves per tile
   int32_t RT;         // T rows per class a tile uses: 128*MH + (Fw-1)/s
   int32_t RA;         // T rows per class allocated (RT rounded up to 8)
@@ -108,9 +110,18 @@ __device__ __forceinline__ bool unit_at(const SParams& P, int64_t it, uint32_t r
     u.store = true;
   }
   const uint32_t img = tile / (uint32_t)P.TPI;
-  u.img = (int32_t)img;
+  u.img = (int32_t)img * P.IPT;
   u.R0 = (int32_t)(tile - img * (uint32_t)P.TPI) * 128 * P.MH;
   return true;
+}
+// T row `rho` of the unit (counted from its image's first) -> the image's number within the tile and the row within that
+// image; whether there is one.
+__device__ __forceinline__ bool row_at(const SParams& P, const Unit& u, int32_t& rho, int32_t& ii) {
+  ii = 0;
+  if (P.IPT == 1) return rho < P.RPI;
+  ii = rho / P.RPI;
+  rho -= ii * P.RPI;
+  return ii < P.IPT && u.img + ii < P.N;
 }
 // Source elements [e_lo, e_hi) of a channel plane that the tile starting at T row R0 needs.
 template <int FH, int S, bool FUSED>
@@ -269,7 +280,15 @@ conv_tc_strip_kernel(const SParams P, const __grid_constant__ CUtensorMap fmap, 
         SPROF_W(0, ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->raw_empty[rr.idx]), rr.phase ^ 1u, DEV_TIMEOUT_RAW_EMPTY, 64))
         if (!ok) break;
         const uint32_t dst0 = raw_sa + (uint32_t)rr.idx * P.raw_stage_bytes;
-        if (P.box) {
+        if (P.IPT > 1) {  // GR consecutive whole planes of each image: one contiguous copy an image
+          if (lane == 0) {
+            const int32_t ni = min(P.IPT, P.N - u.img);
+            const uint32_t bytes = (uint32_t)(P.GR * P.CP) * ES;
+            ptx::mbar_arrive_expect_tx(full, bytes * (uint32_t)ni);
+            for (int32_t i = 0; i < ni; ++i)
+              ptx::bulk_g2s(dst0 + (uint32_t)i * bytes, xsrc + ((int64_t)(u.img + i) * P.C + ch0) * P.plane, bytes, full);
+          }
+        } else if (P.box) {
           if (lane == 0) {
             ptx::mbar_arrive_expect_tx(full, P.raw_stage_bytes);
             tma_load_2d(dst0, &xmap, box_x, u.img * P.C + ch0, full);
@@ -383,21 +402,22 @@ conv_tc_strip_kernel(const SParams P, const __grid_constant__ CUtensorMap fmap, 
         if (task < ntasks) {
           const int32_t cb = task / P.NJ, j = task - cb * P.NJ;
           const int32_t p = j / S, cl = j - p * S;      // T row within the tile, class
-          const int32_t rho = u.R0 + p;
+          int32_t rho = u.R0 + p, ii;
+          const bool row = row_at(P, u, rho, ii);
           const int32_t m = rho / P.WP, q = rho - m * P.WP;
           const int32_t k = q * S + cl;
-          if (rho < P.RPI && k < P.W) {
+          if (row && k < P.W) {
             tv[z] = true;
             tcb[z] = cb;
             const int32_t e = FUSED ? (m * S * P.W + k) : (m * P.W + k) * FH;
-            soff[z] = (uint32_t)(e - e_lo + cb * NCH * P.CP) * ES;
+            soff[z] = (uint32_t)(e - e_lo + (ii * P.GR + cb * NCH) * P.CP) * ES;
             doff[z] = (uint32_t)(cl * P.RA + p) * 16u + (uint32_t)(cb * FH) * lbo;
           }
         }
       }
       // 16-byte phase of the staged ranges: per tile, plus (bulk copies of planes that are not a whole
       // number of chunks) per channel
-      const int32_t sk0 = (int32_t)(((int64_t)u.img * P.C * P.plane + e_lo) & (EPC - 1));
+      const int32_t sk0 = P.IPT > 1 ? 0 : (int32_t)(((int64_t)u.img * P.C * P.plane + e_lo) & (EPC - 1));
       for (int32_t ts = 0; ts < P.NTS && ok; ++ts, tr.advance(2)) {
         const uint32_t t_stage = t_sa + (uint32_t)tr.idx * P.t_stage_bytes;
         for (int32_t sub = 0; sub < P.NSUB && ok; ++sub, rr.advance(P.SR)) {
@@ -466,13 +486,14 @@ conv_tc_strip_kernel(const SParams P, const __grid_constant__ CUtensorMap fmap, 
         hphase ^= 1u;
         ptx::tc_fence_after();
         if (hh < P.MH) {
-          const int32_t rho = u.R0 + hh * 128 + q4 * 32 + lane;
+          int32_t rho = u.R0 + hh * 128 + q4 * 32 + lane, ii;
+          const bool row = row_at(P, u, rho, ii);
           const int32_t m = rho / P.WP, q = rho - m * P.WP;
-          const bool valid = u.store && rho < P.RPI && q < P.Wo;
+          const bool valid = u.store && row && q < P.Wo;
           const int32_t n0 = u.nt * P.NT;
-          const int64_t HoWo = (int64_t)P.Ho * P.Wo;
-          float* const orow = P.nhwc ? P.out + ((int64_t)u.img * HoWo + (int64_t)m * P.Wo + q) * P.K + n0
-                                     : P.out + ((int64_t)u.img * P.K + n0) * HoWo + (int64_t)m * P.Wo + q;
+          const int64_t HoWo = (int64_t)P.Ho * P.Wo, img = u.img + ii;
+          float* const orow = P.nhwc ? P.out + (img * HoWo + (int64_t)m * P.Wo + q) * P.K + n0
+                                     : P.out + (img * P.K + n0) * HoWo + (int64_t)m * P.Wo + q;
           store_columns(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(hh * P.NT), orow, P.nhwc ? 1 : HoWo, P.epi_split, P.NT,
                         P.K - n0, valid, false, P.nhwc && (P.K & 3) == 0);
           ptx::tc_fence_before();
@@ -500,12 +521,14 @@ conv_tc_strip_kernel(const SParams P, const __grid_constant__ CUtensorMap fmap, 
     for (int64_t it = 0; ok; ++it, dr.advance(P.ND)) {
       Unit u;
       if (!unit_at<PAIR>(P, it, rank, u)) break;
-      const int32_t rho = u.R0 + h * 128 + q4 * 32 + lane;
+      int32_t rho = u.R0 + h * 128 + q4 * 32 + lane, ii;
+      const bool row = row_at(P, u, rho, ii);
       const int32_t m = rho / P.WP, q = rho - m * P.WP;
-      const bool valid = u.store && rho < P.RPI && q < P.Wo;
+      const bool valid = u.store && row && q < P.Wo;
       const int32_t n0 = u.nt * P.NT;
-      float* const orow = P.nhwc ? P.out + ((int64_t)u.img * eHoWo + (int64_t)m * P.Wo + q) * eK + n0
-                                 : P.out + ((int64_t)u.img * P.K + n0) * eHoWo + (int64_t)m * P.Wo + q;
+      const int64_t img = u.img + ii;
+      float* const orow = P.nhwc ? P.out + (img * eHoWo + (int64_t)m * P.Wo + q) * eK + n0
+                                 : P.out + (img * P.K + n0) * eHoWo + (int64_t)m * P.Wo + q;
       SPROF_W(0, ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->acc_full[dr.idx]), dr.phase, DEV_TIMEOUT_ACC, 128))
       if (!ok) break;
       ptx::tc_fence_after();
@@ -587,7 +610,7 @@ struct Plan {
 
 // Fills the launch parameters for (FH, FW, S, BF16, SRCK); IM2WIN_EUNSUPPORTED where the kernel does not apply.
 template <int FH, int FW, int S, bool BF16, int SRCK>
-int make_plan(const Geometry& g, Plan* pl, int pair, int mh_fixed) {
+int make_plan(const Geometry& g, Plan* pl, int pair, int mh_fixed, bool images = false) {
   constexpr int NCH = BF16 ? 8 : 4;
   constexpr int64_t ES = SRCK == 2 ? 2 : 4;
   constexpr int64_t EPC = 16 / ES;
@@ -618,7 +641,14 @@ int make_plan(const Geometry& g, Plan* pl, int pair, int mh_fixed) {
   P.MH = mh_fixed;
   if (P.MH * P.NT > 512) return IM2WIN_EUNSUPPORTED;
   P.TPI = (P.RPI + 128 * P.MH - 1) / (128 * P.MH);
-  P.tiles = (int64_t)g.N * P.TPI;
+  P.IPT = 1;
+  P.N = g.N;
+  if (images) {
+    P.IPT = 128 * P.MH / P.RPI;
+    if (P.IPT > g.N) P.IPT = g.N;
+    if (P.IPT < 2) return IM2WIN_EUNSUPPORTED;
+  }
+  P.tiles = images ? (g.N + P.IPT - 1) / P.IPT : (int64_t)g.N * P.TPI;
   P.units = pair ? ((P.tiles + 1) / 2) * P.n_ntiles : P.tiles * P.n_ntiles;
   if (P.tiles * P.n_ntiles >= (1ll << 31) - 65536) return IM2WIN_EUNSUPPORTED;  // (the kernel's unit arithmetic is 32-bit)
   P.RT = 128 * P.MH + SH;
@@ -630,6 +660,10 @@ int make_plan(const Geometry& g, Plan* pl, int pair, int mh_fixed) {
   int64_t cp = len_max + 2 * EPC;
   const int64_t cp_align = 32 / ES;  // a row is a whole number of 32 bytes: a stage of >= 4 rows a whole number of 128
   cp = (cp + cp_align - 1) / cp_align * cp_align;
+  if (images) {  // whole planes, one behind the other
+    cp = P.plane;
+    P.pm = 0;
+  }
   if (cp * ES > 65536) return IM2WIN_EUNSUPPORTED;
   P.CP = (int32_t)cp;
   P.t_stage_bytes = (uint32_t)(GDIV * FH * S * P.RA * 16);
@@ -649,7 +683,8 @@ int make_plan(const Geometry& g, Plan* pl, int pair, int mh_fixed) {
       if (cbn > 1) continue;
     }
     if ((int64_t)P.NJ * cbn > (int64_t)kTMax * kTW * 32) return IM2WIN_EUNSUPPORTED;
-    const int64_t raw_bytes = (int64_t)cbn * NCH * cp * ES;
+    int64_t raw_bytes = (int64_t)cbn * NCH * cp * ES;
+    if (images) raw_bytes = (raw_bytes * P.IPT + 127) / 128 * 128;
     if (cbn * NCH > 32 || raw_bytes % 128 != 0) continue;
     if (2 * (int64_t)P.b_stage_bytes + 2 * raw_bytes > left) continue;
     P.CBN = cbn;
@@ -674,7 +709,7 @@ int make_plan(const Geometry& g, Plan* pl, int pair, int mh_fixed) {
   }
   if (!sb) return IM2WIN_EUNSUPPORTED;
   P.NSUB = P.G / P.GR;
-  P.box = (P.pm == 0 && cp * ES <= 2048 && P.GR >= 4 && encode_fn() != nullptr && (int64_t)g.N * g.C <= INT32_MAX &&
+  P.box = (!images && P.pm == 0 && cp * ES <= 2048 && P.GR >= 4 && encode_fn() != nullptr && (int64_t)g.N * g.C <= INT32_MAX &&
            !knobs().no_box) ? 1 : 0;
   P.SB = (int32_t)sb; P.SR = (int32_t)sr;
   uint32_t off = (uint32_t)(P.SB * P.b_stage_bytes);
@@ -808,12 +843,12 @@ int launch_kernel(const SParams& P, const Plan& pl, const CUtensorMap& fmap, con
 
 template <int FH, int FW, int S, bool BF16, int SRCK>
 int launch_strip(const void* src, const float* f, float* out, const Geometry& g, cudaStream_t st, Scratch scratch,
-                 bool even_if_slower) {
+                 bool even_if_slower, bool images) {
   Plan pl;
-  int rc = choose_plan<FH, FW, S, BF16, SRCK>(g, &pl);
+  int rc = images ? make_plan<FH, FW, S, BF16, SRCK>(g, &pl, 0, 1, true) : choose_plan<FH, FW, S, BF16, SRCK>(g, &pl);
   if (rc != IM2WIN_OK) return rc;
   SParams& P = pl.P;
-  if (!even_if_slower && !knobs().force_strip && !strip_preferred<FH, FW, S, BF16, SRCK>(g, P)) return IM2WIN_EUNSUPPORTED;
+  if (!images && !even_if_slower && !knobs().force_strip && !strip_preferred<FH, FW, S, BF16, SRCK>(g, P)) return IM2WIN_EUNSUPPORTED;
   if (!scratch.ptr || scratch.bytes < pl.scratch_bytes || (reinterpret_cast<uintptr_t>(scratch.ptr) & 15u)) return IM2WIN_EUNSUPPORTED;
   EncodeTiledFn enc = encode_fn();
   if (!enc) return IM2WIN_EUNSUPPORTED;
@@ -862,11 +897,11 @@ template <int FH, int FW, int S>
 int launch_strip_fs(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                     Scratch scratch, int src_kind, bool slow_ok) {
   const bool bf16 = mode == IM2WIN_MODE_BF16;
-  if (src_kind == 2) return bf16 ? launch_strip<FH, FW, S, true, 2>(src, f, out, g, st, scratch, slow_ok) : IM2WIN_EUNSUPPORTED;
-  if (src_kind == 1) return bf16 ? launch_strip<FH, FW, S, true, 1>(src, f, out, g, st, scratch, slow_ok)
-                                 : launch_strip<FH, FW, S, false, 1>(src, f, out, g, st, scratch, slow_ok);
-  return bf16 ? launch_strip<FH, FW, S, true, 0>(src, f, out, g, st, scratch, slow_ok)
-              : launch_strip<FH, FW, S, false, 0>(src, f, out, g, st, scratch, slow_ok);
+  if (src_kind == 2) return bf16 ? launch_strip<FH, FW, S, true, 2>(src, f, out, g, st, scratch, slow_ok, false) : IM2WIN_EUNSUPPORTED;
+  if (src_kind == 1) return bf16 ? launch_strip<FH, FW, S, true, 1>(src, f, out, g, st, scratch, slow_ok, false)
+                                 : launch_strip<FH, FW, S, false, 1>(src, f, out, g, st, scratch, slow_ok, false);
+  return bf16 ? launch_strip<FH, FW, S, true, 0>(src, f, out, g, st, scratch, slow_ok, false)
+              : launch_strip<FH, FW, S, false, 0>(src, f, out, g, st, scratch, slow_ok, false);
 }
 
 template <int FH, int FW, int S>
@@ -889,6 +924,24 @@ int launch_conv_tc_strip(const void* src, const float* f, float* out, const Geom
   if (g.Fh == 3 && g.Fw == 3 && g.s == 1) return launch_strip_fs<3, 3, 1>(src, f, out, g, mode, st, scratch, src_kind, even_if_slower);
   if (g.Fh == 3 && g.Fw == 3 && g.s == 2) return launch_strip_fs<3, 3, 2>(src, f, out, g, mode, st, scratch, src_kind, even_if_slower);
   return IM2WIN_EUNSUPPORTED;
+}
+
+// Several whole images per tile, for 3x3 layers of stride 1 in BF16 mode on images whose T rows (Ho * W) fit a block of 128 at
+// least twice: a tile of one such image computes up to three quarters of its rows for nothing, and as many rounds of units more.
+// Single CTAs, one block: faster than pairs (by 15 % in the mean) and than two blocks.  B200, 160 random calls of this kind, where
+// the gather kernel does not take them: 0.84 of the time, 5 of them slower by more than 3 % (128 images of 512x9x9, 512 filters,
+// transform and convolution 92.7 -> 70.3 us; 69 of 448x6x11, 64 filters, fused 56 -> 31).  Not in TF32 mode (119 calls 1.02), not at
+// stride 2, whose T stages leave the rings too little, and not on deep layers of wide filter tiles whose images are one round of
+// units anyway (32 of 512x9x9, 512 filters, fused: window kernel 45 us, here 51).
+int launch_conv_tc_strip_images(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
+                                Scratch scratch, int src_kind, bool out_bf16) {
+  if (out_bf16 || knobs().strip_images == 2) return IM2WIN_EUNSUPPORTED;
+  if (mode != IM2WIN_MODE_BF16 || g.Fh != 3 || g.Fw != 3 || g.s != 1 || g.N < 2 || (int64_t)g.Ho * g.W > 64) return IM2WIN_EUNSUPPORTED;
+  const int64_t n_nt = (g.K + 255) / 256;
+  if (g.C >= 256 && g.K > 128 * n_nt && g.N * n_nt <= sm_count() && knobs().strip_images != 1) return IM2WIN_EUNSUPPORTED;
+  if (src_kind == 2) return launch_strip<3, 3, 1, true, 2>(src, f, out, g, st, scratch, false, true);
+  if (src_kind == 1) return launch_strip<3, 3, 1, true, 1>(src, f, out, g, st, scratch, false, true);
+  return launch_strip<3, 3, 1, true, 0>(src, f, out, g, st, scratch, false, true);
 }
 
 size_t strip_scratch_bytes(const Geometry& g, int mode, int src_kind) {
