@@ -34,7 +34,7 @@ def _stale() -> bool:
 
 # These files hold families of kernel instantiations (by filter size); compiled as so many translation units
 # (-DIM2WIN_PART=k) they build in parallel.
-PARTS = {"conv_tc_persistent.cu": 8, "conv_tc_window.cu": 2}
+PARTS = {"conv_tc_persistent.cu": 8, "conv_tc_window.cu": 5}
 
 
 def build_library(force: bool = False, verbose: bool = False, out: str | None = None,

@@ -289,6 +289,11 @@ int conv_impl(const void* src, int src_kind, const float* filter, const im2win_s
         r = launch_conv_tc_window(xhat, filter, out_nchw, g, mode, st, sc, 1, out16, /*even_if_slower=*/true);
       return r;
     };
+    // (where this kernel takes a rectangular filter or a channel count of its wider families, it has been compared with the general one)
+    if (general_first && !knobs().force_generic && window_family(g, mode)) {
+      rc = launch_conv_tc_window(xhat, filter, out_nchw, g, mode, st, scratch_from(0), 1, out16);
+      if (rc != IM2WIN_EUNSUPPORTED) return rc;
+    }
     if (general_first) {
       // The general kernel needs no workspace.  But without room for the im2win tensor a call that no fused specialisation
       // takes is refused, and stays refused.
@@ -356,7 +361,11 @@ int im2win_conv_workspace_bytes(const im2win_shape* shape, int src_kind, int mod
   if (mode != IM2WIN_MODE_TF32 && mode != IM2WIN_MODE_BF16 && mode != IM2WIN_MODE_FP32) return IM2WIN_EINVAL;
   const size_t win = src_kind == IM2WIN_SRC_NCHW ? ((size_t)g.n_win * 4 + 255) / 256 * 256 : 0;
   const int kind = src_kind == IM2WIN_SRC_NCHW_FUSED ? 1 : (src_kind == IM2WIN_SRC_IM2WIN_BF16 ? 2 : 0);
-  const size_t extra = conv_scratch_bytes(g, mode, kind);
+  size_t extra = conv_scratch_bytes(g, mode, kind);
+  if (src_kind == IM2WIN_SRC_NCHW) {  // (the window-offset kernel that writes the tensor itself)
+    const size_t own = window_scratch_bytes(g, mode, 3);
+    if (own > extra) extra = own;
+  }
   *bytes = extra ? win + extra : (src_kind == IM2WIN_SRC_NCHW ? (size_t)g.n_win * 4 : 0);
   return IM2WIN_OK;
 }

@@ -76,17 +76,21 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
                    Scratch scratch, int src_kind, bool out_bf16);
 // Scratch bytes with which every kernel above is available for this problem (0 if none wants any).
 size_t strip_scratch_bytes(const Geometry& g, int mode, int src_kind);
-// The window-offset kernel (conv_tc_window.cu; stride 1, 3x3 and 5x5): same source kinds and scratch rules, and kind 3: the
-// untransformed input, the fp32 im2win tensor written to `xhat` beside the result.
+// The window-offset kernel (conv_tc_window.cu; stride 1, 3x3 and 5x5, from the input several rectangular filters too): same source
+// kinds and scratch rules, and kind 3: the untransformed input, the fp32 im2win tensor written to `xhat` beside the result.
 int launch_conv_tc_window(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                           Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower = false, float* xhat = nullptr);
 size_t window_scratch_bytes(const Geometry& g, int mode, int src_kind);
+// Rectangular filters, and channel counts that are no whole filter blocks: taken from the input only, where estimated faster.
+bool window_family(const Geometry& g, int mode);
 // (its plan, for the test build) two issuing threads, resident filter, filter stages; false where not implemented
 bool window_issue_plan(const Geometry& g, int mode, int src_kind, int* two, int* resident, int* stages);
 size_t persistent_scratch_bytes(const Geometry& g, int mode);
 // The gather kernel (conv_tc_gather.cu): fp32 sources (`fused`: the untransformed input), any filter size, fp32 output,
 // no scratch.  behind_transform: what this call has enqueued before is its own transform, which it may overlap.
 bool gather_preferred(const Geometry& g, int mode, bool fused);
+// Its estimated time from the input, in microseconds.
+double gather_us(const Geometry& g, int mode);
 // Whether, from the input, it is expected to beat the transform followed by a specialised kernel on the im2win tensor.
 bool gather_beats_transform(const Geometry& g, int mode);
 int launch_conv_tc_gather(const float* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,

@@ -507,22 +507,25 @@ bool gather_preferred(const Geometry& g, int mode, bool fused) {
   return gather_plan(g, bf16, fused, 256).us < limit;
 }
 
-// For fused calls that no fused specialisation takes (rows whose staged input does not fit shared memory).  The kernel's
-// time: the plan's, and for every wave behind the first the 1.5 + 0.015 NT us of a CTA's start and store that nothing hides
-// there; the other side: the transform, and the persistent kernel as above with an epilogue in every wave.  Fitted to 104
+// Estimated time from the input, in microseconds: the plan's, and for every wave behind the first the 1.5 + 0.015 NT us of a
+// CTA's start and store that nothing hides there.
+double gather_us(const Geometry& g, int mode) {
+  const GPlan pl = gather_plan(g, mode == IM2WIN_MODE_BF16, true, 256);
+  if (pl.NT == 0) return 1e30;
+  const int64_t slots = cluster_slots(pl.Z, sm_count());
+  const int64_t waves = ((g.Mtot + 127) / 128 * pl.n_ntiles * pl.Z + slots - 1) / slots;
+  return pl.us + (double)(waves - 1) * (1.5 + 0.015 * pl.NT);
+}
+
+// For fused calls that no fused specialisation takes (rows whose staged input does not fit shared memory).  The other
+// side: the transform, and the persistent kernel as above with an epilogue in every wave.  Fitted to 104
 // such layers (rows of 400 to 2,600 columns) on B200: the picks take 3 % more than the better of the two on each, the
 // transform and the specialised kernel always 13 %, this kernel always 33 % (1080x1920, 7x7 stride 2 from three channels, 64
 // filters, TF32 141 and 230 us; 64x1600, 3x5, 16 channels, 64 filters 23 and 53; 200x1000, 7x1, 32 channels 221 and 103).
 bool gather_beats_transform(const Geometry& g, int mode) {
-  const bool bf16 = mode == IM2WIN_MODE_BF16;
-  const GPlan pl = gather_plan(g, bf16, true, 256);
-  if (pl.NT == 0) return false;
-  const int64_t nsm = sm_count(), tiles = (g.Mtot + 127) / 128, slots = cluster_slots(pl.Z, (int)nsm);
-  const int64_t waves = (tiles * pl.n_ntiles * pl.Z + slots - 1) / slots;
-  const int64_t n256 = (g.K + 255) / 256, pwaves = (tiles * n256 + nsm - 1) / nsm;
-  const double gather = pl.us + (double)(waves - 1) * (1.5 + 0.015 * pl.NT);
-  const double other = transform_us(g) + persistent_us(g, bf16) + (double)(pwaves - 1) * (double)(g.K / n256) * 0.016;
-  return gather < other;
+  const int64_t nsm = sm_count(), n256 = (g.K + 255) / 256, pwaves = ((g.Mtot + 127) / 128 * n256 + nsm - 1) / nsm;
+  const double other = transform_us(g) + persistent_us(g, mode == IM2WIN_MODE_BF16) + (double)(pwaves - 1) * (double)(g.K / n256) * 0.016;
+  return gather_us(g, mode) < other;
 }
 
 int launch_conv_tc_gather(const float* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,

@@ -75,6 +75,7 @@ struct WParams {
   int32_t two;        // two MMA-issuing threads share the filter stages by parity; every MMA accumulates, the epilogue zeroes behind its reads
   int32_t pair;       // two CTAs (a cluster) work as one: tcgen05.mma.cta_group::2, M = 256, each CTA its own rows and half the filter tile
   int32_t G, GR, NSUB, NXS;  // channels per X stage / per source stage, source stages per X stage, X stages per unit
+  int32_t k_odd;      // the last X stage's last MMA step has no channel: not issued
   int32_t TPS;        // taps per filter stage (Fw: one filter row per stage; 1: one tap per stage)
   int32_t SR, SB, ND;
   int32_t n_epi;      // epilogue warps in use
@@ -150,6 +151,7 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
   Ring xr, br, dr;
   bool ok = true;
   constexpr bool two = TWO;
+  const bool k_odd = P.k_odd != 0;
   const bool bres = P.bres != 0;  // resident filter: the stages of a unit are the ring, filled once
   uint32_t bc = 0;  // filter stages so far: with two issuing threads, thread `which` takes those of its parity
   (void)bc; (void)which;
@@ -205,6 +207,7 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
               for (int blk = 0; blk < NBLK; ++blk) {
 #pragma unroll
                 for (int k2 = 0; k2 < 2; ++k2) {
+                  if (blk == NBLK - 1 && k2 == 1 && k_odd && xs == P.NXS - 1) continue;
                   mma_ss_e<BF16, PAIR>(d_tmem + (uint32_t)h * NT, a_k, a_hi, b_k + (uint32_t)k2 * 2u, b_hi, idesc, acc, elect);
                   acc = 1;
                   a_k += kstep16;
@@ -236,6 +239,10 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
 // 3 = untransformed input, the fp32 im2win tensor written beside the result.
 template <int SRCK>
 constexpr bool kFromInput = SRCK == 1 || SRCK == 3;
+
+// CTA pairs: the square filters only.
+template <int FH, int FW>
+constexpr bool kPairs = FH == FW && (FH == 3 || FH == 5);
 
 template <int FH, int FW, bool BF16, int SRCK, bool PAIR>
 __global__ void __launch_bounds__(SRCK == 3 ? 640 + 32 * kXW : 640, 1)
@@ -330,9 +337,12 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
           continue;
         }
 #endif
-        if (P.dense) {
+        const int32_t nch = min(P.GR, P.C - ch0);  // (the last stages may have channels missing, or all of them)
+        if (nch <= 0) {
+          if (lane == 0) ptx::mbar_arrive(full);
+        } else if (P.dense) {
           if (lane == 0) {
-            const uint32_t bytes = (uint32_t)(P.GR * P.BXE) * ES;
+            const uint32_t bytes = (uint32_t)(nch * P.BXE) * ES;
             ptx::mbar_arrive_expect_tx(full, bytes);
             ptx::bulk_g2s(dst0, xsrc + ((int64_t)u.img * P.C + ch0) * P.plane, bytes, full);
           }
@@ -346,7 +356,7 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
         } else {
           const SrcT* src = nullptr;
           uint32_t dst = 0, bytes = 0;
-          if (lane < P.GR) {
+          if (lane < nch) {
             const int64_t start = ((int64_t)u.img * P.C + ch0 + lane) * P.plane + e_lo;
             const int32_t skew = (int32_t)(start & (EPC - 1));
             const int64_t a0 = start - skew;
@@ -508,6 +518,7 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
           const uint32_t rs = raw_sa + (uint32_t)rr.idx * P.raw_stage_bytes;
           const int32_t ch0 = (xs * P.NSUB + sub) * P.GR;
           const uint32_t x_sub = x_stage + (uint32_t)(sub * ncb) * lbo;
+          const int32_t nch = P.C - ch0;  // channels from here on: the missing ones are zeros
 #pragma unroll
           for (int z = 0; z < kXMax; ++z) {
 #ifdef IM2WIN_PROF
@@ -517,12 +528,14 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
               const uint32_t d0 = x_sub + (uint32_t)(tid + z * (kTW * 32)) * 16u;
               for (int32_t cb = 0; cb < ncb; ++cb) {
                 uint32_t val[NCH];
+                const bool whole = (cb + 1) * NCH <= nch;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
                   const int32_t ch = cb * NCH + c;
                   const int32_t sk = P.pm ? ((sk0 + (ch0 + ch) * P.pm) & (EPC - 1)) : 0;
                   const uint32_t a = rs + soff[z] + (uint32_t)(ch * P.BXE + sk) * ES;
-                  val[c] = SRC16 ? lds_u16(a) : lds_u32(a);
+                  val[c] = 0;
+                  if (whole || ch < nch) val[c] = SRC16 ? lds_u16(a) : lds_u32(a);
                 }
                 const uint32_t d = d0 + (uint32_t)cb * lbo;
                 if constexpr (!BF16) {
@@ -645,7 +658,7 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
         if (!ok) break;
         if (u.store && turn == u.nt) {
           const uint32_t rs = raw_sa + (uint32_t)rr.idx * P.raw_stage_bytes;
-          for (int32_t ch = xw; ch < P.GR; ch += kXW) {
+          for (int32_t ch = xw; ch < min(P.GR, P.C - sidx * P.GR); ch += kXW) {
             const int32_t c = sidx * P.GR + ch;
             const int32_t sk = P.pm ? ((sk0 + c * P.pm) & (EPC - 1)) : sk0;
             uint32_t a = rs + (uint32_t)(ch * P.BXE + sk) * 4u;
@@ -692,22 +705,23 @@ constexpr int kPrepCh = 128, kPrepTaps = 25;
 // first MMA waits for this copy: its latency counts).
 template <bool BF16>
 __global__ void __launch_bounds__(128) filter_image_kernel(const float* __restrict__ f, uint8_t* __restrict__ o, int32_t K, int32_t NT,
-                                                           int32_t NTB, int32_t C, int32_t taps, int32_t TPS, int32_t G) {
+                                                           int32_t NTB, int32_t C, int32_t Cp, int32_t taps, int32_t TPS,
+                                                           int32_t G) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int ES = BF16 ? 2 : 4;
   constexpr int BKE = 64 / ES;  // channels per row
   __shared__ float sm[kPrepCh * kPrepTaps];
   const int32_t j = (int32_t)blockIdx.x, tid = (int32_t)threadIdx.x;
   const int32_t c0 = (int32_t)blockIdx.y * kPrepCh;
-  const int32_t nc = min(kPrepCh, C - c0);
+  const int32_t nc = min(kPrepCh, Cp - c0);
   const float* fj = f + ((int64_t)j * C + c0) * taps;
-  const int32_t n = nc * taps;
+  const int32_t n = nc * taps, nf = min(nc, C - c0) * taps;  // (zeros for the channels of [C, Cp))
   if (j < K) {
     float v[kPrepTaps];
 #pragma unroll
     for (int q = 0; q < kPrepTaps; ++q) {  // (all loads in flight before the first use)
       const int32_t i = tid + q * 128;
-      v[q] = (q < taps && i < n) ? __ldg(fj + i) : 0.f;
+      v[q] = (q < taps && i < nf) ? __ldg(fj + i) : 0.f;
     }
 #pragma unroll
     for (int q = 0; q < kPrepTaps; ++q) {
@@ -722,7 +736,7 @@ __global__ void __launch_bounds__(128) filter_image_kernel(const float* __restri
     const int32_t nt = j / NT, half = (j - nt * NT) / NTB, r = j - nt * NT - half * NTB, ch = c0 + tid, nhalf = NT / NTB;
     const int32_t xs = ch / G, blk = (ch - xs * G) / BKE, cb = (ch % BKE) * ES, nblk = G / BKE, nst = taps / TPS;
     const size_t blk_bytes = (size_t)NTB * 64, tap_bytes = blk_bytes * nblk, stage_bytes = tap_bytes * TPS;
-    uint8_t* d = o + ((size_t)(nt * (C / G) + xs) * nst * nhalf + half) * stage_bytes + blk * blk_bytes +
+    uint8_t* d = o + ((size_t)(nt * (Cp / G) + xs) * nst * nhalf + half) * stage_bytes + blk * blk_bytes +
                  (size_t)((r >> 3) * 512 + (r & 7) * 64 + (((cb >> 4) ^ ((r >> 1) & 3)) << 4) + (cb & 15));
     const size_t skip = (size_t)(nhalf - 1) * stage_bytes;  // the other half's
     for (int32_t t = 0, dt = 1; t < taps; ++t, ++dt, d += tap_bytes) {
@@ -753,7 +767,8 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   P = WParams{};
   if (g.s != 1) return IM2WIN_EUNSUPPORTED;
   const int gmin = 4 * NCH;  // one 64-byte filter block
-  if (g.C % gmin != 0) return IM2WIN_EUNSUPPORTED;
+  const int32_t Cp = (g.C + gmin - 1) / gmin * gmin;
+  if (!kFromInput<SRCK> && Cp != g.C) return IM2WIN_EUNSUPPORTED;
   if (g.HoWo > (1 << 28) || (int64_t)g.H * g.W > (1 << 26)) return IM2WIN_EUNSUPPORTED;
   P.C = g.C; P.K = g.K; P.Ho = g.Ho; P.Wo = g.Wo; P.W = g.W; P.H = g.H;
   P.nhwc = g.out_nhwc;
@@ -844,7 +859,7 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
         if (nblk < 1 || nblk > 2 || (tps != 1 && tps != FW) || gr < NCH) return IM2WIN_EUNSUPPORTED;
       }
       const int G = nblk * gmin;
-      if (g.C % G != 0 || G % gr != 0 || gr > 32 || gr < NCH) continue;
+      if (Cp % G != 0 || G % gr != 0 || gr > 32 || gr < NCH) continue;
       const uint32_t x_stage_bytes = (uint32_t)((G / NCH) * P.RA * 16);
       const int64_t left = cap - 2 * (int64_t)x_stage_bytes;
       const int64_t b_stage_bytes = (int64_t)tps * nblk * blk_bytes;
@@ -863,20 +878,20 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
       // about 100 cycles each, and their slots are sized for 128 rows of any image (9x9, 512 channels: the copies alone
       // took the kernel's 117 kcycles; BF16 from the tensor, with the transform, 101 -> 90 us; 10x10, 128 channels, 64
       // filters, BF16 fused 14.7 -> 13.2, from the tensor 23.2 -> 19.4)
-      const bool dense = P.TPI == 1 && gr % EPC == 0 && P.plane < (1 << 20) && !knobs().no_box;
+      const bool dense = P.TPI == 1 && gr % EPC == 0 && g.C % EPC == 0 && P.plane < (1 << 20) && !knobs().no_box;
       if (dense) { nbx = 1; bxe = P.plane; }
       int64_t raw_bytes = (int64_t)gr * nbx * bxe * ES;
       if (dense) raw_bytes = (raw_bytes + 127) / 128 * 128;
       if (raw_bytes % 128 != 0 || bxe * ES > 65536) continue;
       // Resident filter: a single filter tile whose Fh*Fw*C/G stages all fit beside the X stages and two source
       // stages stays in shared memory for the whole kernel (no filter stream, no release traffic).
-      const int64_t n_res = (int64_t)(g.C / G) * (FH * FW / tps);
+      const int64_t n_res = (int64_t)(Cp / G) * (FH * FW / tps);
       const bool try_res = pass == 0 && n_res <= kMaxB && n_res * b_stage_bytes + 2 * raw_bytes <= left;
       if (pass == 0 && !try_res) continue;
       if (try_res) {
         int64_t sr = 2;
         while (sr < kMaxRaw && n_res * b_stage_bytes + (sr + 1) * raw_bytes <= left) ++sr;
-        P.G = G; P.NXS = g.C / G; P.x_stage_bytes = x_stage_bytes;
+        P.G = G; P.NXS = Cp / G; P.x_stage_bytes = x_stage_bytes;
         P.TPS = tps; P.b_stage_bytes = (uint32_t)b_stage_bytes;
         P.GR = gr; P.NSUB = G / gr; P.dense = dense ? 1 : 0; P.box = box_ok && !dense ? 1 : 0;
         P.NBX = (int32_t)nbx; P.BXE = (int32_t)bxe; P.raw_stage_bytes = (uint32_t)raw_bytes;
@@ -903,7 +918,7 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
         if (can_b && (!can_r || cover_b <= cover_r)) sb += step_b;
         else ++sr;
       }
-      P.G = G; P.NXS = g.C / G; P.x_stage_bytes = x_stage_bytes;
+      P.G = G; P.NXS = Cp / G; P.x_stage_bytes = x_stage_bytes;
       P.TPS = tps; P.b_stage_bytes = (uint32_t)b_stage_bytes;
       P.GR = gr; P.NSUB = nsub; P.dense = dense ? 1 : 0; P.box = box_ok && !dense ? 1 : 0;
       P.NBX = (int32_t)nbx; P.BXE = (int32_t)bxe; P.raw_stage_bytes = (uint32_t)raw_bytes;
@@ -927,7 +942,10 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   P.tmem_cols = 32;
   while ((int32_t)P.tmem_cols < cols) P.tmem_cols *= 2;
   P.idesc = ptx::make_idesc(pair ? 256 : 128, P.NT, BF16 ? 1 : 2);
-  pl->scratch_bytes = (size_t)FH * FW * P.Kp * (size_t)g.C * (BF16 ? 2 : 4);
+  pl->scratch_bytes = (size_t)FH * FW * P.Kp * (size_t)Cp * (BF16 ? 2 : 4);
+  // (channels completed with zeros: within the bound that im2win.h states on the scratch)
+  if (Cp != g.C && pl->scratch_bytes > 8 * (size_t)FH * FW * (g.K > 16 ? g.K : 16) * (size_t)(g.C > 32 ? g.C : 32)) return IM2WIN_EUNSUPPORTED;
+  P.k_odd = Cp - g.C >= 2 * NCH ? 1 : 0;
   pl->threads = (kEpiWarp0 + P.n_epi + (SRCK == 3 ? kXW : 0)) * 32;
   return IM2WIN_OK;
 }
@@ -946,13 +964,14 @@ int choose_wplan(const Geometry& g, WPlan* best) {
   const int forced = knobs().window_mh & 255;
   const int nt = (((g.K + (g.K + 255) / 256 - 1) / ((g.K + 255) / 256)) + 15) / 16 * 16;
   int pair = 0;
-  if (FH == 5) pair = BF16 ? nt >= 256 && (int64_t)g.Ho * g.W >= 640 : kFromInput<SRCK> && nt > 64;  // (BF16: slower on 20x20 outputs)
-  else if (kFromInput<SRCK> && !BF16) pair = nt > 64 && nt <= 128 && g.W >= 60;
+  if (FH == 5 && FW == 5) pair = BF16 ? nt >= 256 && (int64_t)g.Ho * g.W >= 640 : kFromInput<SRCK> && nt > 64;  // (BF16: slower on 20x20 outputs)
+  else if (FH == 3 && FW == 3 && kFromInput<SRCK> && !BF16) pair = nt > 64 && nt <= 128 && g.W >= 60;
   if (knobs().window_pair == 1) pair = 1;
   if (knobs().window_pair == 2) pair = 0;
   WPlan small_pairs;
   bool have_small_pairs = false;
   for (int attempt = 0; attempt < 2; ++attempt, pair = 1 - pair) {
+    if (pair && !kPairs<FH, FW>) { if (knobs().window_pair) break; else continue; }
     if (attempt == 1 && knobs().window_pair) break;  // (a forced variant that does not fit: unsupported)
     double best_cost = -1;
     // a unit's time beside its blocks, in blocks: the halo rows of X and the tile's hand-overs weigh more the fewer
@@ -1044,6 +1063,52 @@ bool xhat_preferred(const Geometry& g, const WParams& P) {
   return here < 0.93 * there;
 }
 
+// Rectangular filters, and channel counts that are no whole filter blocks (completed with zeros), from the untransformed input:
+// against the persistent kernel (behind the transform for kind 3) and, where that would be taken, the gather kernel, all in
+// microseconds.  Fits to 3,100 random calls on B200 (this kernel within 10 % in the median, the persistent kernel within 18 %).
+// Over those calls the picks take 0.86 of the others' time from SRC_NCHW and 0.94 fused, the better of the two on each 0.80 and
+// 0.88; 79 of them are slower than the others by more than 3 %.  Filters without a persistent kernel (3x4) are compared with the
+// gather kernel alone: 0.66 and 0.75, none slower.  (77 images of 64x53x58, 80 3x4 filters, BF16 325 -> 74 us; 39 of 160x22x16, 176
+// 1x7 filters, channels-last 28.5 -> 16.5; 59 of 75x22x22, 48 5x5 filters, fused 46 -> 21.)
+template <int FH, int FW, bool BF16, int SRCK>
+bool family_preferred(const Geometry& g, const WParams& P) {
+  //                                     start  MMAs   rows  columns tensor / channels-last columns  pairs
+  static const double on[2][2][6] = {{{8.5, 1.02, 0.93, 2.27, 0.49, 2.8}, {8.1, 1.01, 1.13, 2.06, 0.31, 1.5}},
+                                     {{8.9, 1.02, 1.20, 1.97, 0.71, 3.8}, {8.5, 1.07, 0.92, 2.10, 0.85, 4.9}}};
+  //                                     start  bytes  steps  steps x columns (streamed)  columns  slices
+  static const double off[2][2][6] = {{{6.1, 0.0, 0.060, 0.029, 1.42, 3.8}, {6.1, 0.0, 0.099, 0.030, 1.45, 3.5}},
+                                      {{9.7, 0.28, 0.038, 0.035, 1.09, 3.1}, {9.8, 0.25, 0.080, 0.035, 1.37, 3.4}}};
+  constexpr bool XHAT = SRCK == 3;
+  const double *a = on[XHAT][BF16], *o = off[XHAT][BF16];
+  if (g.C < 16) return false;
+  const int64_t nsm = sm_count(), slots = P.pair ? nsm / 2 : nsm, rounds = (P.units + slots - 1) / slots, step = BF16 ? 16 : 8;
+  const double mma = FH * FW * (double)((g.C + step - 1) / step) * P.MH * (P.NT > 108 ? P.NT / 2.0 : 54.0) / 1900.0;
+  const double extra = XHAT ? g.C * 128 * P.MH * FH * 4 / P.n_ntiles * 1e-5 : (P.nhwc ? P.NT * P.MH * 0.01 : 0.0);
+  const double here = a[0] + a[5] * P.pair + (double)rounds * (a[1] * mma + a[2] * P.NXS * P.G * (128 * P.MH + (FH - 1) * g.W) * 1e-4 +
+                      a[3] * P.NT * P.MH * 0.01 + a[4] * extra);
+  const double bytes = XHAT ? (double)(g.n_in + g.n_win) * 4e-6 : 0.0;
+  double there = 1e30;
+  if (FH != 3 || FW != 4) {
+    constexpr int64_t FF = FH * FW, CB = FF == 1 ? 32 : (BF16 || FF < 7 ? 16 : 8);
+    const int64_t ng = (g.C + CB - 1) / CB, S = (CB * FF + step - 1) / step;
+    const int64_t tiles = (g.Mtot + 127) / 128 * P.n_ntiles, waves = (tiles + nsm - 1) / nsm;
+    int64_t z = tiles >= nsm || P.nhwc ? 1 : nsm / tiles;
+    z = z > 16 ? 16 : z;
+    z = z > ng ? ng : z;
+    const double steps = (double)(waves * ng * S) / (double)z;
+    const bool resident = P.n_ntiles == 1 && ng * S * P.NT * 32 < 150000;
+    there = o[0] + o[1] * bytes + o[2] * steps + (resident ? 0.0 : o[3] * steps * P.NT * 0.01) +
+            o[4] * (double)waves * P.NT * 0.01 * (P.nhwc ? 2.0 : 1.0) + (z > 1 ? o[5] : 0.0);
+    if (here >= 0.9 * there) return false;
+  }
+  const int mode = BF16 ? IM2WIN_MODE_BF16 : IM2WIN_MODE_TF32;
+  if ((FH == 3 && FW == 4) || gather_preferred(g, mode, true)) {
+    const double gather = gather_us(g, mode) + (XHAT ? 2.0 + 0.12 * bytes : 0.0);  // (it overlaps the transform)
+    if (gather < there) there = gather;
+  }
+  return here < 0.9 * there;
+}
+
 // Whether this kernel is expected to beat the strip-matrix and the persistent kernel: rules read off a
 // measured table (B200, batch 128, every stride-1 3x3 / 5x5 layer of the benchmark lists, three source kinds,
 // both modes).  Its strengths: the staged bytes and the interleaving work are a third of the strip-matrix
@@ -1060,6 +1125,8 @@ bool xhat_preferred(const Geometry& g, const WParams& P) {
 template <int FH, int FW, bool BF16, int SRCK>
 bool window_preferred(const Geometry& g, const WParams& P) {
   const int nsm = sm_count();
+  if constexpr (kFromInput<SRCK>)
+    if (!kPairs<FH, FW> || P.NXS * P.G != g.C) return family_preferred<FH, FW, BF16, SRCK>(g, P);
   if (SRCK == 3) return xhat_preferred<FH, FW, BF16>(g, P);
   if (P.units * 2 <= nsm) return false;  // under-filled launches: the persistent kernel's reduction slices
   if (FH == 5) {  // 25 taps of one staged tile (TF32 from the tensor: smaller images)
@@ -1126,6 +1193,12 @@ int launch_wkernel(const WParams& P, const WPlan& pl, const CUtensorMap& fmap, c
 template <int FH, int FW, bool BF16, int SRCK>
 int launch_window(const void* src, const float* f, float* out, const Geometry& g, cudaStream_t st, Scratch scratch,
                   bool even_if_slower, float* xhat) {
+  // Rectangular filters, and channel counts that are no whole filter blocks: where the general kernel could serve the call too
+  // (what is refused without it stays refused), and only where they are faster.  (Calls below 1e7 multiplications take the time of
+  // their launches whatever the kernel: not looked at.)
+  const bool family = !kPairs<FH, FW> || g.C % (BF16 ? 32 : 16) != 0;
+  if (family && (!scratch.wide || (!knobs().force_window && !even_if_slower && (double)g.n_out * (double)g.Kg < 1e7))) return IM2WIN_EUNSUPPORTED;
+  if (family && SRCK != 3) even_if_slower = false;
   WPlan pl;
   int rc = choose_wplan<FH, FW, BF16, SRCK>(g, &pl);
   if (rc != IM2WIN_OK) return rc;
@@ -1173,10 +1246,14 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
       P.NBX = 1;
     }
   }
-  const dim3 pgrid((unsigned)P.Kp, (unsigned)((g.C + kPrepCh - 1) / kPrepCh));
-  filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, P.NTB, g.C, FH * FW, P.TPS, P.G);
+  const int32_t Cp = P.NXS * P.G;
+  const dim3 pgrid((unsigned)P.Kp, (unsigned)((Cp + kPrepCh - 1) / kPrepCh));
+  filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, P.NTB, g.C, Cp, FH * FW, P.TPS, P.G);
   if (cudaGetLastError() != cudaSuccess) return IM2WIN_ECUDA;
-  rc = P.pair ? launch_wkernel<FH, FW, BF16, SRCK, true>(P, pl, fmap, xmap, st) : launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
+  if constexpr (kPairs<FH, FW>)
+    rc = P.pair ? launch_wkernel<FH, FW, BF16, SRCK, true>(P, pl, fmap, xmap, st) : launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
+  else
+    rc = launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
   if (rc != IM2WIN_OK) return rc;
   note_kernel(KERNEL_WINDOW);
   {
@@ -1198,6 +1275,25 @@ int launch_window_fs(const void* src, const float* f, float* out, const Geometry
   return bf16 ? launch_window<FH, FW, true, 0>(src, f, out, g, st, scratch, eis, nullptr) : launch_window<FH, FW, false, 0>(src, f, out, g, st, scratch, eis, nullptr);
 }
 
+// Rectangular filters: from the untransformed input.
+template <int FH, int FW>
+int launch_window_rect(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st, Scratch scratch,
+                       int src_kind, bool eis, float* xhat) {
+  const bool bf16 = mode == IM2WIN_MODE_BF16;
+  if (src_kind == 3)
+    return bf16 ? launch_window<FH, FW, true, 3>(src, f, out, g, st, scratch, eis, xhat) : launch_window<FH, FW, false, 3>(src, f, out, g, st, scratch, eis, xhat);
+  if (src_kind == 1)
+    return bf16 ? launch_window<FH, FW, true, 1>(src, f, out, g, st, scratch, eis, nullptr) : launch_window<FH, FW, false, 1>(src, f, out, g, st, scratch, eis, nullptr);
+  return IM2WIN_EUNSUPPORTED;
+}
+template <int FH, int FW>
+int wplan_rect(const Geometry& g, int mode, int src_kind, WPlan* pl) {
+  const bool bf16 = mode == IM2WIN_MODE_BF16;
+  if (src_kind == 3) return bf16 ? choose_wplan<FH, FW, true, 3>(g, pl) : choose_wplan<FH, FW, false, 3>(g, pl);
+  if (src_kind == 1) return bf16 ? choose_wplan<FH, FW, true, 1>(g, pl) : choose_wplan<FH, FW, false, 1>(g, pl);
+  return IM2WIN_EUNSUPPORTED;
+}
+
 template <int FH, int FW>
 int wplan_fs(const Geometry& g, int mode, int src_kind, WPlan* pl) {
   const bool bf16 = mode == IM2WIN_MODE_BF16;
@@ -1209,8 +1305,8 @@ int wplan_fs(const Geometry& g, int mode, int src_kind, WPlan* pl) {
 
 }  // namespace
 
-// The filter sizes' kernels build as translation units in parallel (-DIM2WIN_PART=0: 3x3 and everything else, 1: 5x5; without
-// the macro everything is compiled here).
+// The filter sizes' kernels build as translation units in parallel (-DIM2WIN_PART=0: 3x3 and everything else, 1: 5x5, 2 to 4:
+// rectangular filters; without the macro everything is compiled here).
 #ifndef IM2WIN_PART
 #define IM2WIN_PART -1
 #endif
@@ -1218,8 +1314,34 @@ int wplan_fs(const Geometry& g, int mode, int src_kind, WPlan* pl) {
                            Scratch scratch, int src_kind, bool even_if_slower, float* xhat
 #define IM2WIN_WINDOW_PASS src, f, out, g, mode, st, scratch, src_kind, even_if_slower, xhat
 int launch_window_5x5(IM2WIN_WINDOW_ARGS);
+int launch_window_rect_a(IM2WIN_WINDOW_ARGS);
+int launch_window_rect_b(IM2WIN_WINDOW_ARGS);
+int launch_window_rect_c(IM2WIN_WINDOW_ARGS);
 #if IM2WIN_PART == -1 || IM2WIN_PART == 1
 int launch_window_5x5(IM2WIN_WINDOW_ARGS) { return launch_window_fs<5, 5>(IM2WIN_WINDOW_PASS); }
+#endif
+#if IM2WIN_PART == -1 || IM2WIN_PART == 2
+int launch_window_rect_a(IM2WIN_WINDOW_ARGS) {
+  if (g.Fh == 1 && g.Fw == 1) return launch_window_rect<1, 1>(IM2WIN_WINDOW_PASS);
+  if (g.Fh == 1 && g.Fw == 3) return launch_window_rect<1, 3>(IM2WIN_WINDOW_PASS);
+  if (g.Fh == 3 && g.Fw == 1) return launch_window_rect<3, 1>(IM2WIN_WINDOW_PASS);
+  return IM2WIN_EUNSUPPORTED;
+}
+#endif
+#if IM2WIN_PART == -1 || IM2WIN_PART == 3
+int launch_window_rect_b(IM2WIN_WINDOW_ARGS) {
+  if (g.Fh == 1 && g.Fw == 7) return launch_window_rect<1, 7>(IM2WIN_WINDOW_PASS);
+  if (g.Fh == 7 && g.Fw == 1) return launch_window_rect<7, 1>(IM2WIN_WINDOW_PASS);
+  return IM2WIN_EUNSUPPORTED;
+}
+#endif
+#if IM2WIN_PART == -1 || IM2WIN_PART == 4
+int launch_window_rect_c(IM2WIN_WINDOW_ARGS) {
+  if (g.Fh == 3 && g.Fw == 5) return launch_window_rect<3, 5>(IM2WIN_WINDOW_PASS);
+  if (g.Fh == 5 && g.Fw == 3) return launch_window_rect<5, 3>(IM2WIN_WINDOW_PASS);
+  if (g.Fh == 3 && g.Fw == 4) return launch_window_rect<3, 4>(IM2WIN_WINDOW_PASS);
+  return IM2WIN_EUNSUPPORTED;
+}
 #endif
 
 #if IM2WIN_PART == -1 || IM2WIN_PART == 0
@@ -1229,6 +1351,10 @@ static int window_plan(const Geometry& g, int mode, int src_kind, WPlan* pl) {
   if (g.s != 1) return IM2WIN_EUNSUPPORTED;
   if (g.Fh == 3 && g.Fw == 3) return wplan_fs<3, 3>(g, mode, src_kind, pl);
   if (g.Fh == 5 && g.Fw == 5) return wplan_fs<5, 5>(g, mode, src_kind, pl);
+#define IM2WIN_RECT(FH, FW) if (g.Fh == FH && g.Fw == FW) return wplan_rect<FH, FW>(g, mode, src_kind, pl)
+  IM2WIN_RECT(1, 1); IM2WIN_RECT(1, 3); IM2WIN_RECT(3, 1); IM2WIN_RECT(1, 7); IM2WIN_RECT(7, 1);
+  IM2WIN_RECT(3, 5); IM2WIN_RECT(5, 3); IM2WIN_RECT(3, 4);
+#undef IM2WIN_RECT
   return IM2WIN_EUNSUPPORTED;
 }
 
@@ -1239,7 +1365,16 @@ int launch_conv_tc_window(const void* src, const float* f, float* out, const Geo
   if (g.s != 1 || knobs().no_window) return IM2WIN_EUNSUPPORTED;
   if (g.Fh == 3 && g.Fw == 3) return launch_window_fs<3, 3>(IM2WIN_WINDOW_PASS);
   if (g.Fh == 5 && g.Fw == 5) return launch_window_5x5(IM2WIN_WINDOW_PASS);
+  for (auto launch : {launch_window_rect_a, launch_window_rect_b, launch_window_rect_c}) {
+    const int rc = launch(IM2WIN_WINDOW_PASS);
+    if (rc != IM2WIN_EUNSUPPORTED) return rc;
+  }
   return IM2WIN_EUNSUPPORTED;
+}
+
+bool window_family(const Geometry& g, int mode) {
+  const bool square = g.Fh == g.Fw && (g.Fh == 3 || g.Fh == 5);
+  return g.s == 1 && (!square || g.C % (mode == IM2WIN_MODE_BF16 ? 32 : 16) != 0);
 }
 
 size_t window_scratch_bytes(const Geometry& g, int mode, int src_kind) {
