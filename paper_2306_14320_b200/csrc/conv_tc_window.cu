@@ -75,7 +75,6 @@ struct WParams {
   int32_t two;        // two MMA-issuing threads share the filter stages by parity; every MMA accumulates, the epilogue zeroes behind its reads
   int32_t pair;       // two CTAs (a cluster) work as one: tcgen05.mma.cta_group::2, M = 256, each CTA its own rows and half the filter tile
   int32_t G, GR, NSUB, NXS;  // channels per X stage / per source stage, source stages per X stage, X stages per unit
-  int32_t k_odd;      // the last X stage's last MMA step has no channel: not issued
   int32_t TPS;        // taps per filter stage (Fw: one filter row per stage; 1: one tap per stage)
   int32_t SR, SB, ND;
   int32_t n_epi;      // epilogue warps in use
@@ -151,7 +150,6 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
   Ring xr, br, dr;
   bool ok = true;
   constexpr bool two = TWO;
-  const bool k_odd = P.k_odd != 0;
   const bool bres = P.bres != 0;  // resident filter: the stages of a unit are the ring, filled once
   uint32_t bc = 0;  // filter stages so far: with two issuing threads, thread `which` takes those of its parity
   (void)bc; (void)which;
@@ -207,7 +205,6 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
               for (int blk = 0; blk < NBLK; ++blk) {
 #pragma unroll
                 for (int k2 = 0; k2 < 2; ++k2) {
-                  if (blk == NBLK - 1 && k2 == 1 && k_odd && xs == P.NXS - 1) continue;
                   mma_ss_e<BF16, PAIR>(d_tmem + (uint32_t)h * NT, a_k, a_hi, b_k + (uint32_t)k2 * 2u, b_hi, idesc, acc, elect);
                   acc = 1;
                   a_k += kstep16;
@@ -240,17 +237,19 @@ __device__ __forceinline__ void wmma_role(const WParams& P, SBars* bars, SMisc* 
 template <int SRCK>
 constexpr bool kFromInput = SRCK == 1 || SRCK == 3;
 
-// CTA pairs: the square filters only.
+// CTA pairs: the square filters only, and whole filter blocks of channels.
 template <int FH, int FW>
 constexpr bool kPairs = FH == FW && (FH == 3 || FH == 5);
 
-template <int FH, int FW, bool BF16, int SRCK, bool PAIR>
+// TAIL: the channel count is no whole number of filter blocks (kernels of their own: the test cost the others 3 to 15 %).
+template <int FH, int FW, bool BF16, int SRCK, bool PAIR, bool TAIL>
 __global__ void __launch_bounds__(SRCK == 3 ? 640 + 32 * kXW : 640, 1)
 conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap, const __grid_constant__ CUtensorMap xmap) {
   constexpr bool FUSED = kFromInput<SRCK>;
   constexpr bool XHAT = SRCK == 3;
   constexpr bool SRC16 = SRCK == 2;
   static_assert(!SRC16 || BF16, "a 16-bit source feeds the BF16 mode");
+  static_assert(!TAIL || (FUSED && !PAIR), "single CTAs, from the input");
   constexpr uint32_t ES = SRC16 ? 2u : 4u;       // bytes per source element
   constexpr int32_t EPC = SRC16 ? 8 : 4;          // source elements per 16-byte chunk
   constexpr int NCH = BF16 ? 8 : 4;               // channels per 16-byte chunk of X
@@ -337,8 +336,8 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
           continue;
         }
 #endif
-        const int32_t nch = min(P.GR, P.C - ch0);  // (the last stages may have channels missing, or all of them)
-        if (nch <= 0) {
+        const int32_t nch = TAIL ? min(P.GR, P.C - ch0) : P.GR;  // (the last stages may have channels missing, or all of them)
+        if (TAIL && nch <= 0) {
           if (lane == 0) ptx::mbar_arrive(full);
         } else if (P.dense) {
           if (lane == 0) {
@@ -518,7 +517,8 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
           const uint32_t rs = raw_sa + (uint32_t)rr.idx * P.raw_stage_bytes;
           const int32_t ch0 = (xs * P.NSUB + sub) * P.GR;
           const uint32_t x_sub = x_stage + (uint32_t)(sub * ncb) * lbo;
-          const int32_t nch = P.C - ch0;  // channels from here on: the missing ones are zeros
+          const int32_t nch = P.C - ch0;  // (TAIL) channels from here on: the missing ones are zeros
+          (void)nch;
 #pragma unroll
           for (int z = 0; z < kXMax; ++z) {
 #ifdef IM2WIN_PROF
@@ -528,14 +528,13 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
               const uint32_t d0 = x_sub + (uint32_t)(tid + z * (kTW * 32)) * 16u;
               for (int32_t cb = 0; cb < ncb; ++cb) {
                 uint32_t val[NCH];
-                const bool whole = (cb + 1) * NCH <= nch;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
                   const int32_t ch = cb * NCH + c;
                   const int32_t sk = P.pm ? ((sk0 + (ch0 + ch) * P.pm) & (EPC - 1)) : 0;
                   const uint32_t a = rs + soff[z] + (uint32_t)(ch * P.BXE + sk) * ES;
-                  val[c] = 0;
-                  if (whole || ch < nch) val[c] = SRC16 ? lds_u16(a) : lds_u32(a);
+                  if constexpr (TAIL) val[c] = ch < nch ? lds_u32(a) : 0u;
+                  else val[c] = SRC16 ? lds_u16(a) : lds_u32(a);
                 }
                 const uint32_t d = d0 + (uint32_t)cb * lbo;
                 if constexpr (!BF16) {
@@ -658,7 +657,7 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
         if (!ok) break;
         if (u.store && turn == u.nt) {
           const uint32_t rs = raw_sa + (uint32_t)rr.idx * P.raw_stage_bytes;
-          for (int32_t ch = xw; ch < min(P.GR, P.C - sidx * P.GR); ch += kXW) {
+          for (int32_t ch = xw; ch < (TAIL ? min(P.GR, P.C - sidx * P.GR) : P.GR); ch += kXW) {
             const int32_t c = sidx * P.GR + ch;
             const int32_t sk = P.pm ? ((sk0 + c * P.pm) & (EPC - 1)) : sk0;
             uint32_t a = rs + (uint32_t)(ch * P.BXE + sk) * 4u;
@@ -945,7 +944,6 @@ int make_wplan(const Geometry& g, WPlan* pl, int pair, int mh_fixed) {
   pl->scratch_bytes = (size_t)FH * FW * P.Kp * (size_t)Cp * (BF16 ? 2 : 4);
   // (channels completed with zeros: within the bound that im2win.h states on the scratch)
   if (Cp != g.C && pl->scratch_bytes > 8 * (size_t)FH * FW * (g.K > 16 ? g.K : 16) * (size_t)(g.C > 32 ? g.C : 32)) return IM2WIN_EUNSUPPORTED;
-  P.k_odd = Cp - g.C >= 2 * NCH ? 1 : 0;
   pl->threads = (kEpiWarp0 + P.n_epi + (SRCK == 3 ? kXW : 0)) * 32;
   return IM2WIN_OK;
 }
@@ -971,7 +969,7 @@ int choose_wplan(const Geometry& g, WPlan* best) {
   WPlan small_pairs;
   bool have_small_pairs = false;
   for (int attempt = 0; attempt < 2; ++attempt, pair = 1 - pair) {
-    if (pair && !kPairs<FH, FW>) { if (knobs().window_pair) break; else continue; }
+    if (pair && (!kPairs<FH, FW> || g.C % (BF16 ? 32 : 16) != 0)) { if (knobs().window_pair) break; else continue; }
     if (attempt == 1 && knobs().window_pair) break;  // (a forced variant that does not fit: unsupported)
     double best_cost = -1;
     // a unit's time beside its blocks, in blocks: the halo rows of X and the tile's hand-overs weigh more the fewer
@@ -1082,7 +1080,7 @@ bool family_preferred(const Geometry& g, const WParams& P) {
   const double *a = on[XHAT][BF16], *o = off[XHAT][BF16];
   if (g.C < 16) return false;
   const int64_t nsm = sm_count(), slots = P.pair ? nsm / 2 : nsm, rounds = (P.units + slots - 1) / slots, step = BF16 ? 16 : 8;
-  const double mma = FH * FW * (double)((g.C + step - 1) / step) * P.MH * (P.NT > 108 ? P.NT / 2.0 : 54.0) / 1900.0;
+  const double mma = FH * FW * (double)(P.NXS * P.G / step) * P.MH * (P.NT > 108 ? P.NT / 2.0 : 54.0) / 1900.0;
   const double extra = XHAT ? g.C * 128 * P.MH * FH * 4 / P.n_ntiles * 1e-5 : (P.nhwc ? P.NT * P.MH * 0.01 : 0.0);
   const double here = a[0] + a[5] * P.pair + (double)rounds * (a[1] * mma + a[2] * P.NXS * P.G * (128 * P.MH + (FH - 1) * g.W) * 1e-4 +
                       a[3] * P.NT * P.MH * 0.01 + a[4] * extra);
@@ -1147,9 +1145,9 @@ bool window_preferred(const Geometry& g, const WParams& P) {
   return g.C >= 128;                                                    // fp32 im2win tensor
 }
 
-template <int FH, int FW, bool BF16, int SRCK, bool PAIR>
+template <int FH, int FW, bool BF16, int SRCK, bool PAIR, bool TAIL>
 int launch_wkernel(const WParams& P, const WPlan& pl, const CUtensorMap& fmap, const CUtensorMap& xmap, cudaStream_t st) {
-  auto kern = conv_tc_window_kernel<FH, FW, BF16, SRCK, PAIR>;
+  auto kern = conv_tc_window_kernel<FH, FW, BF16, SRCK, PAIR, TAIL>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem) != cudaSuccess) {
     cudaGetLastError();
     return IM2WIN_ECUDA;
@@ -1250,10 +1248,16 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   const dim3 pgrid((unsigned)P.Kp, (unsigned)((Cp + kPrepCh - 1) / kPrepCh));
   filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, P.NTB, g.C, Cp, FH * FW, P.TPS, P.G);
   if (cudaGetLastError() != cudaSuccess) return IM2WIN_ECUDA;
-  if constexpr (kPairs<FH, FW>)
-    rc = P.pair ? launch_wkernel<FH, FW, BF16, SRCK, true>(P, pl, fmap, xmap, st) : launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
-  else
-    rc = launch_wkernel<FH, FW, BF16, SRCK, false>(P, pl, fmap, xmap, st);
+  rc = IM2WIN_EUNSUPPORTED;
+  if constexpr (kFromInput<SRCK>) {
+    // (the rectangular filters have the one kernel for any channel count)
+    if (!kPairs<FH, FW> || Cp != g.C) rc = launch_wkernel<FH, FW, BF16, SRCK, false, true>(P, pl, fmap, xmap, st);
+  }
+  if constexpr (kPairs<FH, FW>) {
+    if (rc == IM2WIN_EUNSUPPORTED)
+      rc = P.pair ? launch_wkernel<FH, FW, BF16, SRCK, true, false>(P, pl, fmap, xmap, st)
+                  : launch_wkernel<FH, FW, BF16, SRCK, false, false>(P, pl, fmap, xmap, st);
+  }
   if (rc != IM2WIN_OK) return rc;
   note_kernel(KERNEL_WINDOW);
   {
