@@ -1150,7 +1150,7 @@ conv_tc_persistent_kernel(const PParams P, const __grid_constant__ CUtensorMap f
 __global__ void __launch_bounds__(256) filter_to_bf16_kernel(const float* __restrict__ f, __nv_bfloat16* __restrict__ o,
                                                              int64_t n) {
   // the convolution kernel that follows may start now (its filter producer waits for this grid's completion)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
     o[i] = __float2bfloat16_rn(f[i]);
 }
@@ -1163,7 +1163,7 @@ __global__ void __launch_bounds__(256) filter_to_bf16_kernel(const float* __rest
 template <typename T>
 __global__ void __launch_bounds__(256) filter_padded_kernel(const float* __restrict__ f, T* __restrict__ o, int32_t Kg,
                                                             int32_t KCG, int32_t KCGP, int32_t NG) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   const int32_t Kgp = NG * KCGP;
   const float* const fj = f + (int64_t)blockIdx.x * Kg;
   T* const oj = o + (int64_t)blockIdx.x * Kgp;
@@ -1474,11 +1474,12 @@ int launch_spec_impl(const void* xhat, const float* f, float* out, const Geometr
       if (pad_copy) {
         const dim3 nb((unsigned)g.K, (unsigned)((row + 1023) / 1024 < 64 ? (row + 1023) / 1024 : 64));
         using CopyT = typename std::conditional<BF16, __nv_bfloat16, float>::type;
-        filter_padded_kernel<CopyT><<<nb, 256, 0, st>>>(f, static_cast<CopyT*>(f_copy), (int32_t)g.Kg, KCG, KCGP, P.NG);
+        if (launch_behind(filter_padded_kernel<CopyT>, dim3(nb), 256, 0, st, f, static_cast<CopyT*>(f_copy), (int32_t)g.Kg, KCG, KCGP, P.NG) != IM2WIN_OK)
+          return IM2WIN_ECUDA;
       } else {
         const int64_t blocks = ((int64_t)g.K * row + 255) / 256;
         const unsigned nb = (unsigned)(blocks < 148 * 8 ? blocks : 148 * 8);
-        filter_to_bf16_kernel<<<nb, 256, 0, st>>>(f, static_cast<__nv_bfloat16*>(f_copy), g.n_flt);
+        if (launch_behind(filter_to_bf16_kernel, dim3(nb), 256, 0, st, f, static_cast<__nv_bfloat16*>(f_copy), g.n_flt) != IM2WIN_OK) return IM2WIN_ECUDA;
       }
       base = f_copy;
     }

@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(128) filter_tap_major_kernel(const float* __re
                                                                int32_t Kp, int32_t C, int32_t FH, int32_t FW) {
   // the convolution kernel that follows may start its prologue now (it waits for this grid's completion
   // before it reads the copy)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   __shared__ float sm[kPrepCh * kPrepFF];
   const int32_t j = (int32_t)blockIdx.x, tid = (int32_t)threadIdx.x;
   const int32_t c0 = (int32_t)blockIdx.y * kPrepCh;
@@ -887,7 +887,8 @@ int launch_strip(const void* src, const float* f, float* out, const Geometry& g,
   {
     static_assert(FH * FW <= kPrepFF, "filter-copy kernel's shared buffer");
     const dim3 pg((unsigned)P.Kp, (unsigned)((g.C + kPrepCh - 1) / kPrepCh));
-    filter_tap_major_kernel<BF16><<<pg, 128, 0, st>>>(f, scratch.ptr, g.K, P.Kp, g.C, FH, FW);
+    rc = launch_behind(filter_tap_major_kernel<BF16>, pg, 128, 0, st, f, scratch.ptr, g.K, P.Kp, g.C, FH, FW);
+    if (rc != IM2WIN_OK) return rc;
   }
   return P.pair ? launch_kernel<FH, FW, S, BF16, SRCK, true>(P, pl, fmap, xmap, st)
                 : launch_kernel<FH, FW, S, BF16, SRCK, false>(P, pl, fmap, xmap, st);

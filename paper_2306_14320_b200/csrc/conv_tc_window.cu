@@ -706,7 +706,7 @@ template <bool BF16>
 __global__ void __launch_bounds__(128) filter_image_kernel(const float* __restrict__ f, uint8_t* __restrict__ o, int32_t K, int32_t NT,
                                                            int32_t NTB, int32_t C, int32_t Cp, int32_t taps, int32_t TPS,
                                                            int32_t G) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   constexpr int ES = BF16 ? 2 : 4;
   constexpr int BKE = 64 / ES;  // channels per row
   __shared__ float sm[kPrepCh * kPrepTaps];
@@ -1197,6 +1197,7 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   const bool family = !kPairs<FH, FW> || g.C % (BF16 ? 32 : 16) != 0;
   if (family && (!scratch.wide || (!knobs().force_window && !even_if_slower && (double)g.n_out * (double)g.Kg < 1e7))) return IM2WIN_EUNSUPPORTED;
   if (family && SRCK != 3) even_if_slower = false;
+  if (family && knobs().no_gather && !knobs().force_window && !even_if_slower) return IM2WIN_EUNSUPPORTED;  // (test build)
   WPlan pl;
   int rc = choose_wplan<FH, FW, BF16, SRCK>(g, &pl);
   if (rc != IM2WIN_OK) return rc;
@@ -1246,8 +1247,9 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   }
   const int32_t Cp = P.NXS * P.G;
   const dim3 pgrid((unsigned)P.Kp, (unsigned)((Cp + kPrepCh - 1) / kPrepCh));
-  filter_image_kernel<BF16><<<pgrid, 128, 0, st>>>(f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, P.NTB, g.C, Cp, FH * FW, P.TPS, P.G);
-  if (cudaGetLastError() != cudaSuccess) return IM2WIN_ECUDA;
+  rc = launch_behind(filter_image_kernel<BF16>, pgrid, 128, 0, st, f, static_cast<uint8_t*>(scratch.ptr), g.K, P.NT, P.NTB, g.C, Cp, FH * FW,
+                     P.TPS, P.G);
+  if (rc != IM2WIN_OK) return rc;
   rc = IM2WIN_EUNSUPPORTED;
   if constexpr (kFromInput<SRCK>) {
     // (the rectangular filters have the one kernel for any channel count)

@@ -55,7 +55,7 @@ template <int FHT>
 __global__ void __launch_bounds__(kThreads) transform_smem_kernel(const TransformParams P) {
   // a convolution launched next as a programmatic dependent may set up (barriers, tensor memory, resident
   // filter) while this grid drains; it waits for this grid's completion before it reads the im2win tensor
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   extern __shared__ __align__(16) float smem[];
   const int32_t Fh = FHT ? FHT : P.Fh;
   const int64_t job = blockIdx.x;
@@ -192,7 +192,7 @@ __device__ __forceinline__ uint16_t bf16_rn(float x) { return (uint16_t)(bf16x2_
 __global__ void __launch_bounds__(kThreads) transform_smem_bf16_kernel(const TransformParams P, uint16_t* out16) {
   // a convolution launched next as a programmatic dependent may set up (barriers, tensor memory, resident
   // filter) while this grid drains; it waits for this grid's completion before it reads the im2win tensor
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   extern __shared__ __align__(16) float smem[];
   const int64_t job = blockIdx.x;
   const int64_t pg = job / P.nblk;
@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(kThreads) transform_gather_bf16_kernel(const f
                                                                           uint16_t* __restrict__ out,
                                                                           int32_t H, int32_t W, int32_t Fh,
                                                                           int32_t s, int32_t Ho, int64_t total) {
+  ptx::pdl_enter();
   const int64_t L = (int64_t)W * Fh;
   for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * kThreads) {
@@ -374,7 +375,7 @@ template <int FH, bool OUT16, int FORM>
 __global__ void __launch_bounds__(kThreads) transform_tile_kernel(const TileParams P) {
   // a convolution launched next as a programmatic dependent may set up (barriers, tensor memory, resident
   // filter) while this grid drains; it waits for this grid's completion before it reads the im2win tensor
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  ptx::pdl_enter();
   using OutT = typename std::conditional<OUT16, uint16_t, float>::type;
   constexpr int32_t OPC = OUT16 ? 8 : 4;  // output elements per 16-byte chunk
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -539,6 +540,7 @@ __global__ void __launch_bounds__(kThreads) transform_gather_kernel(const float*
                                                                      float* __restrict__ out,
                                                                      int32_t H, int32_t W, int32_t Fh,
                                                                      int32_t s, int32_t Ho, int64_t total) {
+  ptx::pdl_enter();
   const int64_t L = (int64_t)W * Fh;
   for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * kThreads) {
@@ -563,8 +565,7 @@ int launch_tile_form(const TileParams& P, int64_t ctas, size_t smem, cudaStream_
     cudaGetLastError();
     return IM2WIN_ECUDA;
   }
-  kern<<<(unsigned)ctas, kThreads, smem, st>>>(P);
-  return cuda_status(cudaGetLastError());
+  return launch_behind(kern, dim3((unsigned)ctas), kThreads, smem, st, P);
 }
 
 template <int FH>
@@ -721,9 +722,8 @@ static int launch_transform_staged(const float* in, float* out, uint16_t* out16,
   if (make_staged_plan(g, &pl) != IM2WIN_OK) {
     const int64_t blocks = (g.n_win + kThreads - 1) / kThreads;
     const int grid = (int)(blocks < 148 * 64 ? blocks : 148 * 64);
-    if (out16) transform_gather_bf16_kernel<<<grid, kThreads, 0, st>>>(in, out16, g.H, g.W, g.Fh, g.s, g.Ho, g.n_win);
-    else transform_gather_kernel<<<grid, kThreads, 0, st>>>(in, out, g.H, g.W, g.Fh, g.s, g.Ho, g.n_win);
-    return cuda_status(cudaGetLastError());
+    return out16 ? launch_behind(transform_gather_bf16_kernel, dim3(grid), kThreads, 0, st, in, out16, g.H, g.W, g.Fh, g.s, g.Ho, g.n_win)
+                 : launch_behind(transform_gather_kernel, dim3(grid), kThreads, 0, st, in, out, g.H, g.W, g.Fh, g.s, g.Ho, g.n_win);
   }
   const size_t smem = pl.smem;
   if (smem > 48 * 1024) {
@@ -741,11 +741,10 @@ static int launch_transform_staged(const float* in, float* out, uint16_t* out16,
   P.magic_L = magic_for((uint32_t)g.L);
   P.magic_Fh = magic_for((uint32_t)g.Fh);
   P.magic_HoL = magic_for((uint32_t)g.HoL);
-  if (out16) transform_smem_bf16_kernel<<<(unsigned)pl.ctas, kThreads, smem, st>>>(P, out16);
-  else if (g.Fh == 7) transform_smem_kernel<7><<<(unsigned)pl.ctas, kThreads, smem, st>>>(P);
-  else if (g.Fh == 11) transform_smem_kernel<11><<<(unsigned)pl.ctas, kThreads, smem, st>>>(P);
-  else transform_smem_kernel<0><<<(unsigned)pl.ctas, kThreads, smem, st>>>(P);
-  return cuda_status(cudaGetLastError());
+  const dim3 grid((unsigned)pl.ctas);
+  if (out16) return launch_behind(transform_smem_bf16_kernel, grid, kThreads, smem, st, P, out16);
+  return launch_behind(g.Fh == 7 ? transform_smem_kernel<7> : (g.Fh == 11 ? transform_smem_kernel<11> : transform_smem_kernel<0>), grid, kThreads,
+                       smem, st, P);
 }
 
 int launch_transform(const float* in, float* out, const Geometry& g, cudaStream_t st) {
