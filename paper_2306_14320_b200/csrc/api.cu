@@ -435,7 +435,7 @@ int im2win_debug_set_option(const char* name, int value) {
       {"no_box", &Knobs::no_box}, {"no_pim", &Knobs::no_pim}, {"bslice", &Knobs::bslice},
       {"no_bslice", &Knobs::no_bslice}, {"splitk", &Knobs::splitk}, {"force_stream", &Knobs::force_stream},
       {"nsets", &Knobs::nsets}, {"no_l2ahead", &Knobs::no_l2ahead}, {"no_btma", &Knobs::no_btma},
-      {"ntiles", &Knobs::ntiles}, {"transform_gather", &Knobs::transform_gather},
+      {"ntiles", &Knobs::ntiles}, {"transform_gather", &Knobs::transform_gather}, {"transform_pairs", &Knobs::transform_pairs},
       {"test_skip_copy", &Knobs::test_skip_copy}, {"strip_mh", &Knobs::strip_mh}, {"strip_images", &Knobs::strip_images}, {"strip_pair", &Knobs::strip_pair},
       {"force_window", &Knobs::force_window}, {"no_window", &Knobs::no_window}, {"window_mh", &Knobs::window_mh},
       {"window_plan", &Knobs::window_plan}, {"window_pair", &Knobs::window_pair}, {"window_two", &Knobs::window_two}, {"window_xhat", &Knobs::window_xhat}, {"no_gather", &Knobs::no_gather}, {"gather_nt", &Knobs::gather_nt}, {"gather_z", &Knobs::gather_z}, {"gather_big", &Knobs::gather_big}, {"gather_zfail", &Knobs::gather_zfail}, {"window_nohelp", &Knobs::window_nohelp}, {"window_bres", &Knobs::window_bres}, {"transform_budget_kb", &Knobs::transform_budget_kb}};

@@ -326,7 +326,97 @@ __device__ __forceinline__ float lds_f32(uint32_t a) {
   return v;
 }
 __device__ __forceinline__ void sts_f32(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void sts_u16(uint32_t a, uint16_t v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(v) : "memory"); }
+
+// What a CTA of the tile transforms works on: npl whole consecutive planes, or mb output rows of one plane.
+template <int FH>
+struct TileJob {
+  int32_t npl, mb, plane_floats, n_in, out_plane, n_out;
+  int64_t src0, dst0;  // first element of the input and of the output range
+  __device__ __forceinline__ explicit TileJob(const TileParams& P) {
+    const int64_t job = blockIdx.x;
+    const int64_t pg = job / P.nblk;
+    const int32_t b = (int32_t)(job - pg * P.nblk);
+    const bool whole = P.nblk == 1;
+    const int64_t plane0 = pg * P.PB;
+    npl = whole ? (int32_t)min((int64_t)P.PB, P.planes - plane0) : 1;
+    const int32_t m0 = b * P.MB;
+    mb = whole ? P.Ho : min(P.MB, P.Ho - m0);
+    const int32_t rows_in = whole ? P.H : (mb - 1) * P.s + FH;
+    plane_floats = rows_in * P.W;
+    n_in = npl * plane_floats;
+    out_plane = mb * P.L;
+    n_out = npl * out_plane;
+    src0 = plane0 * P.HW + (int64_t)m0 * P.s * P.W;
+    dst0 = plane0 * P.HoL + (int64_t)m0 * P.L;
+  }
+};
+
+// The job's input range in shared memory (element e of it at tin0[skew + e]); false where the copy did not come.
+__device__ __forceinline__ bool stage_input(const TileParams& P, int64_t src0, int32_t n_in, float* tin0, uint64_t* bar, int32_t& skew) {
+  // ---- input range -> shared memory (one bulk copy of the enclosing aligned range)
+  skew = (int32_t)(src0 & 3);                                     // P.in is 16-byte aligned
+  const int64_t a0 = src0 - skew;
+  int32_t nfl = (skew + n_in + 3) & ~3;
+  int32_t ntail = 0;                                              // floats past the last whole chunk
+  if (a0 + nfl > P.n_in_total) {                                  // the last chunk would pass the tensor's end
+    nfl = (int32_t)((P.n_in_total - a0) & ~(int64_t)3);
+    ntail = (int32_t)(P.n_in_total - a0) - nfl;
+  }
+  const uint32_t bar_a = ptx::smem_u32(bar);
+  if (threadIdx.x == 0) {
+    ptx::mbar_init(bar_a, 1);
+    ptx::fence_mbar_init();
+    ptx::mbar_arrive_expect_tx(bar_a, (uint32_t)nfl * 4u);
+    // (test hook: with test_skip_copy the copy is announced but never issued, so that the expiry
+    // path of the bounded wait below can be exercised by a kernel that neither faults nor hangs)
+    if (nfl > 0 && !P.test_skip_copy) ptx::bulk_g2s(ptx::smem_u32(tin0), P.in + a0, (uint32_t)nfl * 4u, bar_a);
+  }
+  if ((int32_t)threadIdx.x < ntail) tin0[nfl + threadIdx.x] = __ldg(P.in + a0 + nfl + threadIdx.x);
+  __syncthreads();  // the barrier is initialised for everyone; the tail floats are in place
+  {
+    // bounded wait: about a second by the global timer (and an iteration cap), then report and leave
+    bool landed = ptx::mbar_try_wait(bar_a, 0u);
+    uint64_t t0 = 0;
+    for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) {
+      __nanosleep(64);
+      landed = ptx::mbar_try_wait(bar_a, 0u);
+      if ((it & 63u) == 63u && !landed) {
+        uint64_t now;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > 1000000000ull) break;
+      }
+    }
+    if (!__all_sync(0xffffffffu, landed)) {
+      if ((threadIdx.x & 31) == 0) atomicCAS(P.status, 0, (int32_t)DEV_TIMEOUT_COPY);
+      return false;
+    }
+  }
+  return true;
+}
+
+// The transposed range (element e of it at tout[e], its 16-byte phase kept) to the output.
+template <typename OutT>
+__device__ __forceinline__ void store_output(const TileParams& P, int64_t dst0, int32_t n_out, OutT* tout, int32_t dskew) {
+  constexpr int32_t OPC = 16 / (int32_t)sizeof(OutT);
+  ptx::fence_proxy_async_smem();  // the buffer is about to be read by the bulk copy
+  __syncthreads();
+
+  // ---- output buffer -> global: one bulk copy of the aligned part, threads for the ragged ends
+  const int32_t head = min((OPC - dskew) & (OPC - 1), n_out);
+  const int32_t nvec = (n_out - head) / OPC;
+  const int32_t tail0 = head + nvec * OPC;
+  OutT* const gout = reinterpret_cast<OutT*>(P.out) + dst0;
+  if (threadIdx.x == 0 && nvec > 0) {
+    ptx::bulk_s2g(gout + head, ptx::smem_u32(tout + head), (uint32_t)nvec * 16u);
+    ptx::bulk_s2g_commit();
+  }
+  if ((int32_t)threadIdx.x < head) gout[threadIdx.x] = tout[threadIdx.x];
+  if ((int32_t)threadIdx.x < n_out - tail0) gout[tail0 + threadIdx.x] = tout[tail0 + threadIdx.x];
+  if (threadIdx.x == 0 && nvec > 0) ptx::bulk_s2g_wait_read();  // shared memory must outlive the copy's reads
+}
 
 // The transposition where rows have an odd length (and FH is odd): every strip starts at another 16-byte phase, so quads
 // of columns would read and write element by element, four lanes to a bank.  A thread takes one column instead:
@@ -383,64 +473,14 @@ __global__ void __launch_bounds__(kThreads) transform_tile_kernel(const TilePara
   OutT* const tout0 = reinterpret_cast<OutT*>(smem_raw + P.off_out);
   uint64_t* const bar = reinterpret_cast<uint64_t*>(smem_raw + P.off_bar);
 
-  const int64_t job = blockIdx.x;
-  const int64_t pg = job / P.nblk;
-  const int32_t b = (int32_t)(job - pg * P.nblk);
-  const bool whole = P.nblk == 1;
-  const int64_t plane0 = pg * P.PB;
-  const int32_t npl = whole ? (int32_t)min((int64_t)P.PB, P.planes - plane0) : 1;
-  const int32_t m0 = b * P.MB;
-  const int32_t mb = whole ? P.Ho : min(P.MB, P.Ho - m0);
-  const int32_t rows_in = whole ? P.H : (mb - 1) * P.s + FH;
-  const int32_t plane_floats = rows_in * P.W;
-  const int32_t n_in = npl * plane_floats;
-  const int32_t out_plane = mb * P.L;
-  const int32_t n_out = npl * out_plane;
-
-  // ---- input range -> shared memory (one bulk copy of the enclosing aligned range)
-  const int64_t src0 = plane0 * P.HW + (int64_t)m0 * P.s * P.W;  // first float of the range
-  const int32_t skew = (int32_t)(src0 & 3);                      // P.in is 16-byte aligned
+  const TileJob<FH> j(P);
+  const int32_t npl = j.npl, mb = j.mb, plane_floats = j.plane_floats, n_in = j.n_in, out_plane = j.out_plane, n_out = j.n_out;
+  int32_t skew;
+  if (!stage_input(P, j.src0, n_in, tin0, bar, skew)) return;
   const float* const tin = tin0 + skew;                           // tin[e] <-> in[src0 + e]
-  const int64_t a0 = src0 - skew;
-  int32_t nfl = (skew + n_in + 3) & ~3;
-  int32_t ntail = 0;                                              // floats past the last whole chunk
-  if (a0 + nfl > P.n_in_total) {                                  // the last chunk would pass the tensor's end
-    nfl = (int32_t)((P.n_in_total - a0) & ~(int64_t)3);
-    ntail = (int32_t)(P.n_in_total - a0) - nfl;
-  }
-  const uint32_t bar_a = ptx::smem_u32(bar);
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(bar_a, 1);
-    ptx::fence_mbar_init();
-    ptx::mbar_arrive_expect_tx(bar_a, (uint32_t)nfl * 4u);
-    // (test hook: with test_skip_copy the copy is announced but never issued, so that the expiry
-    // path of the bounded wait below can be exercised by a kernel that neither faults nor hangs)
-    if (nfl > 0 && !P.test_skip_copy) ptx::bulk_g2s(ptx::smem_u32(tin0), P.in + a0, (uint32_t)nfl * 4u, bar_a);
-  }
-  if ((int32_t)threadIdx.x < ntail) tin0[nfl + threadIdx.x] = __ldg(P.in + a0 + nfl + threadIdx.x);
-  __syncthreads();  // the barrier is initialised for everyone; the tail floats are in place
-  {
-    // bounded wait: about a second by the global timer (and an iteration cap), then report and leave
-    bool landed = ptx::mbar_try_wait(bar_a, 0u);
-    uint64_t t0 = 0;
-    for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) {
-      __nanosleep(64);
-      landed = ptx::mbar_try_wait(bar_a, 0u);
-      if ((it & 63u) == 63u && !landed) {
-        uint64_t now;
-        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
-        if (t0 == 0) t0 = now;
-        else if (now - t0 > 1000000000ull) break;
-      }
-    }
-    if (!__all_sync(0xffffffffu, landed)) {
-      if ((threadIdx.x & 31) == 0) atomicCAS(P.status, 0, (int32_t)DEV_TIMEOUT_COPY);
-      return;
-    }
-  }
 
   // ---- transpose shared -> shared
-  const int64_t dst0 = plane0 * P.HoL + (int64_t)m0 * P.L;       // first element of the output range
+  const int64_t dst0 = j.dst0;
   const int32_t dskew = (int32_t)(dst0 & (OPC - 1));              // P.out is 16-byte aligned
   OutT* const tout = tout0 + dskew;                               // tout[e] <-> out[dst0 + e]
   const int32_t sW = P.s * P.W;
@@ -517,21 +557,53 @@ __global__ void __launch_bounds__(kThreads) transform_tile_kernel(const TilePara
       }
     }
   }
-  ptx::fence_proxy_async_smem();  // the buffer is about to be read by the bulk copy
-  __syncthreads();
+  store_output<OutT>(P, dst0, n_out, tout, dskew);
+}
 
-  // ---- output buffer -> global: one bulk copy of the aligned part, threads for the ragged ends
-  const int32_t head = min((OPC - dskew) & (OPC - 1), n_out);
-  const int32_t nvec = (n_out - head) / OPC;
-  const int32_t tail0 = head + nvec * OPC;
-  OutT* const gout = reinterpret_cast<OutT*>(P.out) + dst0;
-  if (threadIdx.x == 0 && nvec > 0) {
-    ptx::bulk_s2g(gout + head, ptx::smem_u32(tout + head), (uint32_t)nvec * 16u);
-    ptx::bulk_s2g_commit();
+// bf16 storage, odd FH: a thread takes two neighbouring columns, 2*FH floats in and FH 32-bit words out.  Neighbouring lanes
+// write FH words apart (an odd number: no bank conflicts) and read two floats apart (two wavefronts a load); quads of columns
+// wrote 16 bits at a time wherever a strip starts at an odd element, four lanes to a bank.  Such a strip's pairs start at an
+// odd column, its first column is a unit of its own.  (B200: 250 random calls of transform and convolution 0.95 of the time, none
+// more than 4 % slower; 128 images of 96x31x31 under five rows, with the convolution 167.8 -> 161.8 us.)
+template <int FH>
+__global__ void __launch_bounds__(kThreads) transform_pairs_kernel(const TileParams P) {
+  ptx::pdl_enter();
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  float* const tin0 = reinterpret_cast<float*>(smem_raw);
+  uint16_t* const tout0 = reinterpret_cast<uint16_t*>(smem_raw + P.off_out);
+  uint64_t* const bar = reinterpret_cast<uint64_t*>(smem_raw + P.off_bar);
+  const TileJob<FH> j(P);
+  int32_t skew;
+  if (!stage_input(P, j.src0, j.n_in, tin0, bar, skew)) return;
+  const int32_t dskew = (int32_t)(j.dst0 & 7);
+  const uint32_t tin_a = ptx::smem_u32(tin0) + (uint32_t)skew * 4u, tout_a = ptx::smem_u32(tout0);
+  const int32_t W = P.W, sW = P.s * W, units_plane = j.mb * P.QW, nunits = j.npl * units_plane;
+  for (int32_t q = threadIdx.x; q < nunits; q += kThreads) {
+    int32_t pl = 0, rem = q;
+    if (j.npl > 1) {
+      pl = (int32_t)(((uint64_t)(uint32_t)q * P.magic_MQ) >> 32);
+      rem = q - pl * units_plane;
+    }
+    const int32_t mm = (int32_t)(((uint64_t)(uint32_t)rem * P.magic_QW) >> 32);
+    const int32_t row = dskew + pl * j.out_plane + mm * P.L;       // the strip's first element in the output buffer
+    const int32_t c = 2 * (rem - mm * P.QW) - (row & 1);           // the pair's first column
+    const uint32_t src = tin_a + (uint32_t)(pl * j.plane_floats + mm * sW + c) * 4u, dst = tout_a + (uint32_t)(row + c * FH) * 2u;
+    float r[2 * FH];
+    if (c >= 0 && c + 1 < W) {
+#pragma unroll
+      for (int u = 0; u < FH; ++u) {
+        r[u] = lds_f32(src + (uint32_t)(u * W) * 4u);
+        r[FH + u] = lds_f32(src + (uint32_t)(u * W + 1) * 4u);
+      }
+#pragma unroll
+      for (int i = 0; i < FH; ++i) sts_u32(dst + (uint32_t)i * 4u, bf16x2_rn(r[2 * i], r[2 * i + 1]));
+    } else if (c < W) {  // one column: the first (c = -1) or the last
+      const uint32_t o = c < 0 ? 1u : 0u;
+#pragma unroll
+      for (int u = 0; u < FH; ++u) sts_u16(dst + (o * FH + u) * 2u, bf16_rn(lds_f32(src + (uint32_t)(u * W) * 4u + o * 4u)));
+    }
   }
-  if ((int32_t)threadIdx.x < head) gout[threadIdx.x] = tout[threadIdx.x];
-  if ((int32_t)threadIdx.x < n_out - tail0) gout[tail0 + threadIdx.x] = tout[tail0 + threadIdx.x];
-  if (threadIdx.x == 0 && nvec > 0) ptx::bulk_s2g_wait_read();  // shared memory must outlive the copy's reads
+  store_output<uint16_t>(P, j.dst0, j.n_out, tout0 + dskew, dskew);
 }
 
 // Fallback for rows too long to stage (Fh*W floats beyond the shared-memory budget): one thread
@@ -671,6 +743,72 @@ int launch_transform_tile(const float* in, void* out, bool out16, const Geometry
   }
 }
 
+// The pairs kernel's jobs: as the tile kernel's, for ranges of 4 bytes in and 2 out.
+int make_pairs_plan(const Geometry& g, TilePlan* pl) {
+  if (g.Fh != 3 && g.Fh != 5 && g.Fh != 7 && g.Fh != 11) return IM2WIN_EUNSUPPORTED;
+  const int64_t planes = (int64_t)g.N * g.C, hw = (int64_t)g.H * g.W, whole = hw * 4 + g.HoL * 2;
+  int64_t budget = 34 * 1024 - 256;
+  if (whole <= 28 * 1024 - 256) budget = 28 * 1024 - 256;
+  if (knobs().transform_budget_kb) budget = (int64_t)knobs().transform_budget_kb * 1024 - 256;  // (test build)
+  int32_t PB = 1, MB = g.Ho, nblk = 1;
+  if (whole <= budget) {
+    PB = (int32_t)(budget / whole);
+    const int64_t want_ctas = 148 * 8;  // keep enough CTAs to fill the machine
+    if (planes / PB < want_ctas) PB = (int32_t)(planes / want_ctas > 0 ? planes / want_ctas : 1);
+  } else {
+    const int64_t mbmax = (budget - (int64_t)(g.Fh - g.s) * g.W * 4) / ((int64_t)g.s * g.W * 4 + (int64_t)g.L * 2);
+    if (mbmax < 1) return IM2WIN_EUNSUPPORTED;
+    MB = (int32_t)(mbmax < g.Ho ? mbmax : g.Ho);
+    nblk = (g.Ho + MB - 1) / MB;
+    MB = (g.Ho + nblk - 1) / nblk;  // balance the blocks
+    if ((int64_t)(g.Fh - g.s) * 4 > (int64_t)(MB - 1) * g.s + g.Fh) return IM2WIN_EUNSUPPORTED;  // (rows read twice)
+  }
+  const int64_t ctas = nblk == 1 ? (planes + PB - 1) / PB : planes * nblk;
+  if (ctas > INT32_MAX) return IM2WIN_EUNSUPPORTED;
+  const int32_t rows_in = nblk == 1 ? g.H : (MB - 1) * g.s + g.Fh;
+  const int64_t in_floats = (int64_t)PB * rows_in * g.W + 8, out_words = (int64_t)PB * (nblk == 1 ? g.HoL : (int64_t)MB * g.L) + 8;
+  pl->P = TileParams{};
+  TileParams& P = pl->P;
+  P.H = g.H; P.W = g.W; P.s = g.s; P.Ho = g.Ho; P.L = g.L;
+  P.MB = MB; P.nblk = nblk; P.PB = PB;
+  P.QW = g.W / 2 + 1;
+  P.planes = planes; P.HW = hw; P.HoL = g.HoL; P.n_in_total = g.n_in;
+  const int64_t units_plane = (int64_t)(nblk == 1 ? g.Ho : MB) * P.QW;
+  if (units_plane * PB * units_plane >= ((int64_t)1 << 32)) return IM2WIN_EUNSUPPORTED;  // reciprocal division exact
+  P.magic_QW = magic_for((uint32_t)P.QW);
+  P.magic_MQ = magic_for((uint32_t)units_plane);
+  P.off_out = (uint32_t)((in_floats * 4 + 127) / 128 * 128);
+  P.off_bar = P.off_out + (uint32_t)((out_words * 2 + 15) / 16 * 16);
+  pl->smem = P.off_bar + 16;
+  pl->ctas = ctas;
+  return IM2WIN_OK;
+}
+
+template <int FH>
+int launch_pairs_fh(const TilePlan& pl, cudaStream_t st) {
+  auto kern = transform_pairs_kernel<FH>;
+  if (pl.smem > 48 * 1024 &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem) != cudaSuccess) {
+    cudaGetLastError();
+    return IM2WIN_ECUDA;
+  }
+  return launch_behind(kern, dim3((unsigned)pl.ctas), kThreads, pl.smem, st, pl.P);
+}
+
+int launch_transform_pairs(const float* in, uint16_t* out, const Geometry& g, cudaStream_t st) {
+  TilePlan pl;
+  if (knobs().transform_pairs == 2) return IM2WIN_EUNSUPPORTED;
+  const int rc = make_pairs_plan(g, &pl);
+  if (rc != IM2WIN_OK) return rc;
+  pl.P.in = in; pl.P.out = out;
+  pl.P.status = device_status_word();
+  if (!pl.P.status) return IM2WIN_ECUDA;
+  if (g.Fh == 3) return launch_pairs_fh<3>(pl, st);
+  if (g.Fh == 5) return launch_pairs_fh<5>(pl, st);
+  if (g.Fh == 7) return launch_pairs_fh<7>(pl, st);
+  return launch_pairs_fh<11>(pl, st);
+}
+
 struct StagedPlan {
   int32_t MB, nblk, PB;
   int64_t ctas;
@@ -760,7 +898,9 @@ int launch_transform(const float* in, float* out, const Geometry& g, cudaStream_
 int launch_transform_bf16(const float* in, uint16_t* out, const Geometry& g, cudaStream_t st) {
   {
     if (!knobs().transform_gather) {
-      const int rc = launch_transform_tile(in, out, true, g, st);
+      int rc = launch_transform_pairs(in, out, g, st);
+      if (rc != IM2WIN_EUNSUPPORTED) return rc;
+      rc = launch_transform_tile(in, out, true, g, st);
       if (rc != IM2WIN_EUNSUPPORTED) return rc;
     }
   }
