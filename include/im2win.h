@@ -78,7 +78,7 @@ int im2win_workspace_bytes(const im2win_shape* shape, size_t* bytes);
 /* Workspace with which im2win_conv can pick its fastest kernel for (shape, src_kind, mode) (no
  * counterpart in the paper): the im2win tensor where src_kind is NCHW (as above, rounded up to 256
  * bytes), plus room for a re-laid-out copy of the filter that some tensor-core kernels stream by TMA
- * (tap-major orders for the strip-matrix and window-offset kernels; bf16 for BF16 mode; rows padded to the
+ * (tap-major orders for the strip-matrix and window-offset kernels, channels completed with zeros; bf16 for BF16 mode; rows padded to the
  * channel groups that do not divide C).  That copy stays below 2 x 4*K'*C'*Fh*Fw bytes, K' the larger of K and 16, C'
  * the larger of C and 32 (most often it is at most the filter's own size), i.e. a few MB against an im2win tensor of tens to hundreds
  * of MB.  A smaller workspace is legal (down to im2win_workspace_bytes, or none for the other source
@@ -112,9 +112,9 @@ int im2win_transform_bf16(const float* in_nchw, const im2win_shape* shape, uint1
  *   O[i][j][m][n] = sum_{r,u,v} Ihat[i][r][m][(n*s+v)*Fh+u] * F[j][r][u][v].
  * (Algorithm 2 prints the strip offset as n*s*Wf+v*Hf+u, which equals the above for Hf==Wf and
  * is the form consistent with Algorithm 1 otherwise.)
- * src:       device.  src_kind NCHW: the input I (N*C*H*W floats); the call first runs the
- *            transform into `workspace`, which then holds Ihat and may be reused by the caller (the
- *            convolution reads Ihat or, where that is faster, the input itself: the same values).
+ * src:       device.  src_kind NCHW: the input I (N*C*H*W floats); the call runs the
+ *            transform into `workspace`, which then holds Ihat and may be reused by the caller (first, or,
+ *            where that is faster, in the convolution kernel itself, which then reads the input: the same values).
  *            src_kind IM2WIN: an im2win tensor; `workspace` may be NULL, or give scratch (see below).
  *            src_kind NCHW_FUSED: the input I; the tensor-core kernel stages the input rows a tile
  *            needs and reads the windows from them, so nothing of size Ihat is written (workspace
