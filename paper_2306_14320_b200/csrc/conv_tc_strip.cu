@@ -505,6 +505,26 @@ conv_tc_strip_kernel(const SParams P, const __grid_constant__ CUtensorMap fmap, 
           }
         }
       }
+      // Behind the CTA's last unit nothing is left to do here: these warps store their share of its columns.
+      if (ok && P.epi_split == P.NT && last_unit<PAIR>(P, it)) {
+        const int32_t set = (warp - kTWarp0) >> 2, q4 = warp & 3, hh = P.MH == 2 ? set : 0;
+        const int32_t buf = P.ND == 2 ? (int32_t)it & 1 : 0;
+        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->acc_full[buf]), (P.ND == 2 ? (uint32_t)it >> 1 : (uint32_t)it) & 1u, DEV_TIMEOUT_ACC, 128);
+        if (!ok) break;
+        ptx::tc_fence_after();
+        int32_t c0, c1;
+        tail_columns(P.NT, P.MH, set + 1, c0, c1);
+        int32_t rho = u.R0 + hh * 128 + q4 * 32 + lane, ii;
+        const bool row = row_at(P, u, rho, ii);
+        const int32_t m = rho / P.WP, q = rho - m * P.WP;
+        const bool valid = u.store && row && q < P.Wo;
+        const int32_t n0 = u.nt * P.NT;
+        const int64_t HoWo = (int64_t)P.Ho * P.Wo, img = u.img + ii;
+        float* const orow = P.nhwc ? P.out + (img * HoWo + (int64_t)m * P.Wo + q) * P.K + n0
+                                   : P.out + (img * P.K + n0) * HoWo + (int64_t)m * P.Wo + q;
+        store_columns(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)((buf * P.MH + hh) * P.NT), orow, P.nhwc ? 1 : HoWo, c0, c1,
+                      P.K - n0, valid, false, P.nhwc && (P.K & 3) == 0);
+      }
     }
     if (warp == kTWarp0) { SPROF_DUMP(2) }
   } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + n_epi_warps) {
@@ -529,11 +549,13 @@ conv_tc_strip_kernel(const SParams P, const __grid_constant__ CUtensorMap fmap, 
       const int64_t img = u.img + ii;
       float* const orow = P.nhwc ? P.out + (img * eHoWo + (int64_t)m * P.Wo + q) * eK + n0
                                  : P.out + (img * P.K + n0) * eHoWo + (int64_t)m * P.Wo + q;
+      int32_t c_begin, c_end = P.epi_split;
+      if (P.epi_split == P.NT && last_unit<PAIR>(P, it)) tail_columns(P.NT, P.MH, 0, c_begin, c_end);
       SPROF_W(0, ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->acc_full[dr.idx]), dr.phase, DEV_TIMEOUT_ACC, 128))
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t d_tmem = tmem_base + lane_base + (uint32_t)((dr.idx * P.MH + h) * P.NT);
-      store_columns(d_tmem, orow, P.nhwc ? 1 : eHoWo, 0, P.epi_split, eK - n0, valid, false, P.nhwc && (eK & 3) == 0);
+      store_columns(d_tmem, orow, P.nhwc ? 1 : eHoWo, 0, c_end, eK - n0, valid, false, P.nhwc && (eK & 3) == 0);
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) {

@@ -202,6 +202,23 @@ __device__ __forceinline__ void store_columns(uint32_t d_tmem, float* orow, int6
   if (zero_behind) ptx::tmem_wait_st();
 }
 
+// Whether iteration `it` is this CTA's (pair's) last unit.
+template <bool PAIR, class PT>
+__device__ __forceinline__ bool last_unit(const PT& P, int64_t it) {
+  return (blockIdx.x >> (PAIR ? 1 : 0)) + ((uint32_t)it + 1u) * (gridDim.x >> (PAIR ? 1 : 0)) >= (uint32_t)P.units;
+}
+
+// Columns [c0, c1) of a CTA's last unit that one share of its warps stores: share 0 the epilogue warps, 1 and 2 the two sets of four
+// warps that built the MMAs' operand, which are idle by then.  Two blocks per tile: each set takes the upper half of one block's
+// columns; one block: three thirds.  (Nothing overlaps the last unit's stores, and layers of one unit per CTA have no other: 128
+// images of 512x9x9, 512 filters, BF16: 15 of 73 kcycles.)
+__device__ __forceinline__ void tail_columns(int32_t NT, int32_t MH, int32_t share, int32_t& c0, int32_t& c1) {
+  const int32_t third = (NT / 3 + 15) / 16 * 16, half = (NT / 2 + 15) / 16 * 16;
+  const int32_t two_thirds = 2 * third < NT ? 2 * third : NT;
+  if (MH == 2) { c0 = share ? half : 0; c1 = share ? NT : half; }
+  else { c0 = share == 0 ? 0 : (share == 1 ? third : two_thirds); c1 = share == 0 ? third : (share == 1 ? two_thirds : NT); }
+}
+
 // ---- host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
