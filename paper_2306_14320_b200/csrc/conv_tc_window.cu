@@ -596,7 +596,11 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
       if (ok && P.epi_split == P.NT && last_unit<PAIR>(P, it)) {
         const int32_t set = (warp - kTWarp0) >> 2, q4 = warp & 3, hh = P.MH == 2 ? set : 0;
         const int32_t buf = P.ND == 2 ? (int32_t)it & 1 : 0;
-        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->acc_full[buf]), (P.ND == 2 ? (uint32_t)it >> 1 : (uint32_t)it) & 1u, DEV_TIMEOUT_ACC, 128);
+        // (They wait for the release of the unit's last X stage, which is committed behind all of the unit's MMAs and of which they
+        // have seen every phase: they see no phase of the accumulator's own barrier but this one, and would take the phase before for
+        // it while that is still open.)
+        const uint32_t li = (uint32_t)xr.idx ^ 1u, lp = xr.phase ^ (li & 1u);  // the stage filled last, and its phase
+        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->t_empty[li]), lp, DEV_TIMEOUT_ACC, 128);
         if (!ok) break;
         ptx::tc_fence_after();
         int32_t c0, c1;
