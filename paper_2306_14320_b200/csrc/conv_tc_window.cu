@@ -465,7 +465,6 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
     bool ok = true;
     SPROF_DECL
     const uint32_t x_full_lead0 = remote ? mapa(ptx::smem_u32(&bars->t_full[0]), 0) : ptx::smem_u32(&bars->t_full[0]);
-    uint32_t hphase = 0;  // (epilogue help) phase of the single accumulator buffer's "full" barrier
     for (int64_t it = 0; ok; ++it) {
       WUnit u;
       if (!wunit_at<PAIR>(P, it, rank, u)) break;
@@ -565,24 +564,31 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
           }
         }
       }
-      // One accumulator buffer: the next unit's MMAs cannot start before this unit's results are stored, so
-      // this warp stores the upper columns of its TMEM lane quarter meanwhile.
-      if (ok && P.epi_split < P.NT) {
-        const int32_t hh = (warp - kTWarp0) >> 2, q4 = warp & 3;
-        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->acc_full[0]), hphase, DEV_TIMEOUT_ACC, 128);
+      // These warps store columns too.  One accumulator buffer: the next unit's MMAs cannot start before this unit's results are
+      // stored, so they take the upper columns of every unit.  Two: their share of the CTA's last unit, behind which nothing is left
+      // to do here.  Either way they wait for the release of the unit's last X stage, which is committed behind all of the unit's
+      // MMAs and of which they have seen every phase.  (Not for the accumulator's own barrier: whoever has skipped a phase of
+      // that takes the one before for this one where it is still open.)
+      const bool every = P.epi_split < P.NT;
+      if (ok && (every || last_unit<PAIR>(P, it))) {
+        const uint32_t li = (uint32_t)xr.idx ^ 1u, lp = xr.phase ^ (li & 1u);  // the stage filled last, and its phase
+        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->t_empty[li]), lp, DEV_TIMEOUT_ACC, 128);
         if (!ok) break;
-        hphase ^= 1u;
         ptx::tc_fence_after();
-        if (hh < P.MH) {
-          const int32_t rho = u.R0 + hh * 128 + q4 * 32 + lane;
-          const int32_t m = rho / P.W, q = rho - m * P.W;
-          const bool valid = u.store && rho < P.RPI && q < P.Wo;
-          const int32_t n0 = u.nt * P.NT;
-          const int64_t HoWo = (int64_t)P.Ho * P.Wo;
-          float* const orow = P.nhwc ? P.out + ((int64_t)u.img * HoWo + (int64_t)m * P.Wo + q) * P.K + n0
-                                     : P.out + ((int64_t)u.img * P.K + n0) * HoWo + (int64_t)m * P.Wo + q;
-          store_columns(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(hh * P.NT), orow, P.nhwc ? 1 : HoWo, P.epi_split, P.NT,
-                        P.K - n0, valid, P.two != 0, P.nhwc && (P.K & 3) == 0);
+        const int32_t set = (warp - kTWarp0) >> 2, q4 = warp & 3, hh = P.MH == 2 ? set : 0;
+        int32_t c0 = P.epi_split, c1 = P.NT;
+        if (!every) tail_columns(P.NT, P.MH, set + 1, c0, c1);
+        const int32_t rho = u.R0 + hh * 128 + q4 * 32 + lane;
+        const int32_t m = rho / P.W, q = rho - m * P.W;
+        const bool valid = u.store && rho < P.RPI && q < P.Wo;
+        const int32_t n0 = u.nt * P.NT;
+        const int64_t HoWo = (int64_t)P.Ho * P.Wo;
+        float* const orow = P.nhwc ? P.out + ((int64_t)u.img * HoWo + (int64_t)m * P.Wo + q) * P.K + n0
+                                   : P.out + ((int64_t)u.img * P.K + n0) * HoWo + (int64_t)m * P.Wo + q;
+        const int32_t buf = P.ND == 2 ? (int32_t)it & 1 : 0;
+        store_columns(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)((buf * P.MH + hh) * P.NT), orow, P.nhwc ? 1 : HoWo, c0, c1,
+                      P.K - n0, valid, every && P.two != 0, P.nhwc && (P.K & 3) == 0);
+        if (every) {
           ptx::tc_fence_before();
           __syncwarp();
           if (lane == 0) {
@@ -591,29 +597,6 @@ conv_tc_window_kernel(const WParams P, const __grid_constant__ CUtensorMap fmap,
             else ptx::mbar_arrive(ae);
           }
         }
-      }
-      // Behind the CTA's last unit nothing is left to do here: these warps store their share of its columns.
-      if (ok && P.epi_split == P.NT && last_unit<PAIR>(P, it)) {
-        const int32_t set = (warp - kTWarp0) >> 2, q4 = warp & 3, hh = P.MH == 2 ? set : 0;
-        const int32_t buf = P.ND == 2 ? (int32_t)it & 1 : 0;
-        // (They wait for the release of the unit's last X stage, which is committed behind all of the unit's MMAs and of which they
-        // have seen every phase: they see no phase of the accumulator's own barrier but this one, and would take the phase before for
-        // it while that is still open.)
-        const uint32_t li = (uint32_t)xr.idx ^ 1u, lp = xr.phase ^ (li & 1u);  // the stage filled last, and its phase
-        ok = wait_bar_warp(P, misc, ptx::smem_u32(&bars->t_empty[li]), lp, DEV_TIMEOUT_ACC, 128);
-        if (!ok) break;
-        ptx::tc_fence_after();
-        int32_t c0, c1;
-        tail_columns(P.NT, P.MH, set + 1, c0, c1);
-        const int32_t rho = u.R0 + hh * 128 + q4 * 32 + lane;
-        const int32_t m = rho / P.W, q = rho - m * P.W;
-        const bool valid = u.store && rho < P.RPI && q < P.Wo;
-        const int32_t n0 = u.nt * P.NT;
-        const int64_t HoWo = (int64_t)P.Ho * P.Wo;
-        float* const orow = P.nhwc ? P.out + ((int64_t)u.img * HoWo + (int64_t)m * P.Wo + q) * P.K + n0
-                                   : P.out + ((int64_t)u.img * P.K + n0) * HoWo + (int64_t)m * P.Wo + q;
-        store_columns(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)((buf * P.MH + hh) * P.NT), orow, P.nhwc ? 1 : HoWo, c0, c1,
-                      P.K - n0, valid, false, P.nhwc && (P.K & 3) == 0);
       }
     }
     if (warp == kTWarp0) { SPROF_DUMP(2) }
