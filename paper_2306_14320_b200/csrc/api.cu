@@ -419,12 +419,12 @@ int im2win_debug_window_plan(const im2win_shape* shape, int src_kind, int mode, 
   const int kind = src_kind == IM2WIN_SRC_NCHW_FUSED ? 1 : (src_kind == IM2WIN_SRC_IM2WIN_BF16 ? 2 : 0);
   return window_issue_plan(g, mode, kind, out3, out3 + 1, out3 + 2) ? IM2WIN_OK : IM2WIN_EUNSUPPORTED;
 }
-// Test build only, no device needed: the transform's tile plan (transform_tile_plan), and the meaning of a status word.
-int im2win_debug_tile_plan(const im2win_shape* shape, int out16, int64_t* out11) {
+// Test build only, no device needed: the transform's plan (transform_tile_plan), and the meaning of a status word.
+int im2win_debug_tile_plan(const im2win_shape* shape, int kind, int64_t* out11) {
   Geometry g;
   const int rc = make_geometry(shape, &g);
   if (rc != IM2WIN_OK) return rc;
-  return transform_tile_plan(g, out16 != 0, out11) ? IM2WIN_OK : IM2WIN_EUNSUPPORTED;
+  return transform_tile_plan(g, kind, out11) ? IM2WIN_OK : IM2WIN_EUNSUPPORTED;
 }
 int im2win_debug_status_of_word(int32_t word) { return status_of_word(word); }
 int im2win_debug_set_option(const char* name, int value) {

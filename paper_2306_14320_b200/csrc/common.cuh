@@ -47,8 +47,9 @@ int launch_transform(const float* in, float* out, const Geometry& g, cudaStream_
 int launch_transform_bf16(const float* in, uint16_t* out, const Geometry& g, cudaStream_t st);
 // Estimated time of the transform, in microseconds.
 double transform_us(const Geometry& g);
-// (the tile kernel's plan, for the test build: MB, nblk, PB, QW, column form, two reciprocals, off_out, off_bar, bytes, CTAs)
-bool transform_tile_plan(const Geometry& g, bool out16, int64_t* v11);
+// (for the test build; kind 0 = the tile kernel's plan, 1 = that for bf16 storage, 2 = the pairs kernel's: MB, nblk, PB, QW, column
+// form, two reciprocals, off_out, off_bar, bytes, CTAs)
+bool transform_tile_plan(const Geometry& g, int kind, int64_t* v11);
 int launch_conv_fp32(const float* xhat, const float* f, float* out, const Geometry& g, cudaStream_t st);
 // Device memory from the caller's workspace (beyond the im2win tensor) that a tensor-core convolution
 // may use for a re-laid-out copy of the filter; ptr may be null / bytes 0 (kernels that need such a

@@ -721,7 +721,8 @@ int make_tile_plan(const Geometry& g, bool out16, TilePlan* pl) {
   P.off_bar = P.off_out + (uint32_t)((out_floats * (out16 ? 2 : 4) + 15) / 16 * 16);
   pl->smem = P.off_bar + 16;
   pl->ctas = ctas;
-  return IM2WIN_OK;
+  // (one block per plane stages the whole plane: under a stride far above Fh that is many rows beyond those it reads)
+  return pl->smem > kMaxDynamicSmem ? IM2WIN_EUNSUPPORTED : IM2WIN_OK;
 }
 
 int launch_transform_tile(const float* in, void* out, bool out16, const Geometry& g, cudaStream_t st) {
@@ -781,7 +782,8 @@ int make_pairs_plan(const Geometry& g, TilePlan* pl) {
   P.off_bar = P.off_out + (uint32_t)((out_words * 2 + 15) / 16 * 16);
   pl->smem = P.off_bar + 16;
   pl->ctas = ctas;
-  return IM2WIN_OK;
+  // (one block per plane stages the whole plane: under a stride far above Fh that is many rows beyond those it reads)
+  return pl->smem > kMaxDynamicSmem ? IM2WIN_EUNSUPPORTED : IM2WIN_OK;
 }
 
 template <int FH>
@@ -918,9 +920,9 @@ double transform_us(const Geometry& g) {
   return 4.0 + out / 1.0;
 }
 
-bool transform_tile_plan(const Geometry& g, bool out16, int64_t* v) {
+bool transform_tile_plan(const Geometry& g, int kind, int64_t* v) {
   TilePlan pl;
-  if (make_tile_plan(g, out16, &pl) != IM2WIN_OK) return false;
+  if ((kind == 2 ? make_pairs_plan(g, &pl) : make_tile_plan(g, kind == 1, &pl)) != IM2WIN_OK) return false;
   const TileParams& P = pl.P;
   const int64_t w[] = {P.MB, P.nblk, P.PB, P.QW, P.cols, (int64_t)P.magic_QW, (int64_t)P.magic_MQ, P.off_out, P.off_bar, (int64_t)pl.smem, pl.ctas};
   for (size_t i = 0; i < sizeof(w) / sizeof(w[0]); ++i) v[i] = w[i];

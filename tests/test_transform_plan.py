@@ -83,6 +83,78 @@ def test_every_index_of_the_tile_transform_stays_in_its_range(out16):
     assert forms.count(True) > 200 and forms.count(False) > 200
 
 
+def _far_strides():
+    """Strides far above the filter: one block per plane stages many rows that it does not read."""
+    rng = random.Random(5)
+    shapes = [(1, 2, 102, 1000, 3, 100), (1, 2, 34, 1900, 3, 32), (2, 3, 60, 700, 5, 90), (1, 1, 300, 300, 7, 299), (3, 4, 41, 90, 11, 30)]
+    for _ in range(600):
+        fh, s = rng.choice((1, 2, 3, 4, 5, 7, 11)), rng.randint(6, 300)
+        shapes.append((rng.randint(1, 9), rng.randint(1, 30), fh + rng.randint(0, 2 * s), rng.choice((rng.randint(1, 60), rng.randint(1, 2500))), fh, s))
+    return shapes
+
+
+def _walk_pairs(shape):
+    """The pairs kernel's plan; whether it takes the shape."""
+    n, c, h, w, fh, s = shape
+    v = (ctypes.c_int64 * 11)()
+    rc = b.lib().im2win_debug_tile_plan(ctypes.byref(b.Shape(n, c, h, w, 1, fh, 1, s)), 2, v)
+    if rc != b.OK:
+        assert rc == b.EUNSUPPORTED
+        return False
+    mb_max, nblk, pb, qw, _, magic_qw, magic_mq, off_out, off_bar, smem, ctas = v
+    ho, row_out = (h - fh) // s + 1, w * fh
+    whole, planes = nblk == 1, n * c
+    assert fh in (3, 5, 7, 11) and qw == w // 2 + 1
+    assert off_out % 128 == 0 and off_bar % 16 == 0 and smem >= off_bar + 8 and smem <= 227 * 1024
+    assert ctas == (-(-planes // pb) if whole else planes * nblk)
+    if whole:
+        assert mb_max == ho
+        jobs = {(min(pb, planes), ho), ((planes - 1) % pb + 1, ho)}
+    else:
+        assert pb == 1 and (nblk - 1) * mb_max < ho <= nblk * mb_max
+        jobs = {(1, mb_max), (1, ho - (nblk - 1) * mb_max)}
+    for npl, mb in jobs:
+        rows_in = h if whole else (mb - 1) * s + fh
+        n_in, n_out = npl * rows_in * w, npl * mb * row_out
+        units_plane = mb * qw
+        q = np.arange(npl * units_plane, dtype=np.uint64)
+        pl = (q * np.uint64(magic_mq)) >> np.uint64(32) if npl > 1 else np.zeros_like(q)
+        rem = q - pl * np.uint64(units_plane)
+        mm = (rem * np.uint64(magic_qw)) >> np.uint64(32)
+        assert npl == 1 or int(q[-1]) * magic_mq < 2 ** 64
+        assert np.array_equal(pl, q // np.uint64(units_plane)) and np.array_equal(mm, rem // np.uint64(qw))
+        pl, mm, k = (a.astype(np.int64) for a in (pl, mm, rem - mm * np.uint64(qw)))
+        for phase in (0, 1):  # of the job's output range; the strips' phases follow
+            row = phase + pl * mb * row_out + mm * row_out
+            first = 2 * k - (row & 1)
+            lo, hi = np.maximum(first, 0), np.minimum(first + 1, w - 1)  # the columns it takes, none where hi < lo
+            took = hi >= lo
+            columns = (pl * mb + mm)[took] * w
+            seen = np.concatenate([columns + lo[took], (columns + hi[took])[hi[took] > lo[took]]])
+            assert np.array_equal(np.sort(seen), np.arange(npl * mb * w))  # every column of every strip once
+            src = (pl * rows_in * w + mm * s * w)[took]
+            assert int((src + lo[took]).min()) >= 0 and int((src + (fh - 1) * w + hi[took]).max()) < n_in
+            pair = hi > lo
+            assert not ((row + first * fh)[pair & took] & 1).any()  # 32-bit stores
+        for skew in range(4):
+            assert ((skew + n_in + 3) & ~3) * 4 <= off_out
+        assert off_out + (7 + n_out) * 2 <= off_bar
+    return True
+
+
+def test_every_index_of_the_pairs_transform_stays_in_its_range():
+    assert sum(_walk_pairs(shape) for shape in _shapes() if shape[4] in (3, 5, 7, 11)) > 500
+
+
+def test_strides_far_above_the_filter():
+    """What a plan accepts fits shared memory; what it declines is another kernel's."""
+    for shape in _far_strides():
+        for out16 in (0, 1):
+            _walk(shape, out16)
+        if shape[4] in (3, 5, 7, 11):
+            _walk_pairs(shape)
+
+
 def test_a_failed_index_check_is_an_error():
     of = b.lib().im2win_debug_status_of_word
     assert of(0) == b.OK
