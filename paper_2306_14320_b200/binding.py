@@ -180,6 +180,16 @@ def last_kernel() -> int:
     return lib().im2win_debug_last_kernel()
 
 
+TRANSFORM_NONE, TRANSFORM_TILE, TRANSFORM_PAIRS, TRANSFORM_STAGED, TRANSFORM_ELEMENT = 0, 1, 2, 3, 4
+
+
+def last_transform() -> int:
+    """Test build only: which transform kernel was launched since the last look (TRANSFORM_*)."""
+    if not _use_test:
+        raise RuntimeError("the test library only: call use_test_library(True) first")
+    return lib().im2win_debug_last_transform()
+
+
 def conv_workspace_bytes(shape, src_kind: int, mode: int) -> int:
     """im2win_conv_workspace_bytes: the workspace with which im2win_conv can use its fastest kernel."""
     b = ctypes.c_size_t()

@@ -115,6 +115,8 @@ const Knobs& knobs() {
 
 static std::atomic<int> g_last_kernel{KERNEL_NONE};
 void note_kernel(int which) { g_last_kernel.store(which, std::memory_order_relaxed); }
+static std::atomic<int> g_last_transform{0};
+void note_transform(int which) { g_last_transform.store(which, std::memory_order_relaxed); }
 static std::atomic<int> g_last_plan[8];
 void note_plan(const int* v, int n) {
   for (int i = 0; i < 8; ++i) g_last_plan[i].store(i < n ? v[i] : 0, std::memory_order_relaxed);
@@ -404,6 +406,8 @@ int im2win_last_device_status(void* cuda_stream, int32_t* status) {
 #ifdef IM2WIN_TEST_KNOBS
 // Test build only: which convolution kernel the last call launched (KERNEL_* of common.cuh).
 int im2win_debug_last_kernel(void) { return g_last_kernel.load(std::memory_order_relaxed); }
+// Test build only: which transform kernel the last transform launched (note_transform); reading it clears it.
+int im2win_debug_last_transform(void) { return g_last_transform.exchange(0, std::memory_order_relaxed); }
 
 // Test build only (libim2win_test.so): set one diagnostic switch by name.  Returns IM2WIN_EINVAL for
 // an unknown name.

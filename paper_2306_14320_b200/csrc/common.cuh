@@ -175,6 +175,8 @@ const Knobs& knobs();
 // test build exposes as im2win_debug_last_kernel; the product library only writes it).
 enum : int { KERNEL_NONE = 0, KERNEL_STRIP = 1, KERNEL_PERSISTENT = 2, KERNEL_FP32 = 4, KERNEL_WINDOW = 5, KERNEL_GATHER = 6 };
 void note_kernel(int which);
+// The transform kernel a call took: 1 = tile, 2 = pairs of columns, 3 = staged gather, 4 = per element.
+void note_transform(int which);
 // The launch plan of the last strip-matrix / window-offset launch (same diagnostic): up to eight integers.
 void note_plan(const int* v, int n);
 

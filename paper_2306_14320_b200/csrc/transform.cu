@@ -353,8 +353,11 @@ struct TileJob {
   }
 };
 
-// The job's input range in shared memory (element e of it at tin0[skew + e]); false where the copy did not come.
-__device__ __forceinline__ bool stage_input(const TileParams& P, int64_t src0, int32_t n_in, float* tin0, uint64_t* bar, int32_t& skew) {
+// The job's input range in shared memory (element e of it at tin0[skew + e]); false where the copy did not come, or where a thread
+// comes with `fine` false (CHECKED).
+template <bool CHECKED = false>
+__device__ __forceinline__ bool stage_input(const TileParams& P, int64_t src0, int32_t n_in, float* tin0, uint64_t* bar, int32_t& skew,
+                                            bool fine = true) {
   // ---- input range -> shared memory (one bulk copy of the enclosing aligned range)
   skew = (int32_t)(src0 & 3);                                     // P.in is 16-byte aligned
   const int64_t a0 = src0 - skew;
@@ -374,7 +377,9 @@ __device__ __forceinline__ bool stage_input(const TileParams& P, int64_t src0, i
     if (nfl > 0 && !P.test_skip_copy) ptx::bulk_g2s(ptx::smem_u32(tin0), P.in + a0, (uint32_t)nfl * 4u, bar_a);
   }
   if ((int32_t)threadIdx.x < ntail) tin0[nfl + threadIdx.x] = __ldg(P.in + a0 + nfl + threadIdx.x);
-  __syncthreads();  // the barrier is initialised for everyone; the tail floats are in place
+  // the barrier is initialised for everyone; the tail floats are in place
+  if constexpr (CHECKED) fine = __syncthreads_and(fine);
+  else __syncthreads();
   {
     // bounded wait: about a second by the global timer (and an iteration cap), then report and leave
     bool landed = ptx::mbar_try_wait(bar_a, 0u);
@@ -394,7 +399,10 @@ __device__ __forceinline__ bool stage_input(const TileParams& P, int64_t src0, i
       return false;
     }
   }
-  return true;
+  if constexpr (CHECKED) {
+    if (!fine && threadIdx.x == 0) atomicCAS(P.status, 0, (int32_t)DEV_RANGE);
+  }
+  return fine;
 }
 
 // The transposed range (element e of it at tout[e], its 16-byte phase kept) to the output.
@@ -573,11 +581,22 @@ __global__ void __launch_bounds__(kThreads) transform_pairs_kernel(const TilePar
   uint16_t* const tout0 = reinterpret_cast<uint16_t*>(smem_raw + P.off_out);
   uint64_t* const bar = reinterpret_cast<uint64_t*>(smem_raw + P.off_bar);
   const TileJob<FH> j(P);
-  int32_t skew;
-  if (!stage_input(P, j.src0, j.n_in, tin0, bar, skew)) return;
   const int32_t dskew = (int32_t)(j.dst0 & 7);
-  const uint32_t tin_a = ptx::smem_u32(tin0) + (uint32_t)skew * 4u, tout_a = ptx::smem_u32(tout0);
   const int32_t W = P.W, sW = P.s * W, units_plane = j.mb * P.QW, nunits = j.npl * units_plane;
+  // The index check, by one thread of a warp that issues no copy: every index of the loop follows from two quotients, and one taken
+  // by a rounded-up reciprocal is off, if anywhere, for the largest numerator that is one below a multiple of the divisor too, which
+  // is the job's last unit and a plane's last; and both ranges lie in their buffers.  A job that fails it is recorded, not copied.
+  // (By every thread for its every unit it took 2 to 6 % of transform and convolution.)
+  bool fine = true;
+  if (threadIdx.x == 32) {
+    const int32_t last_pl = j.npl > 1 ? (int32_t)(((uint64_t)(uint32_t)(nunits - 1) * P.magic_MQ) >> 32) : 0;
+    const int32_t last_mm = (int32_t)(((uint64_t)(uint32_t)(units_plane - 1) * P.magic_QW) >> 32);
+    fine = last_pl == j.npl - 1 && last_mm == j.mb - 1 && (uint32_t)(3 + j.n_in) * 4u <= P.off_out &&
+           P.off_out + (uint32_t)(dskew + j.n_out) * 2u <= P.off_bar;
+  }
+  int32_t skew;
+  if (!stage_input<true>(P, j.src0, j.n_in, tin0, bar, skew, fine)) return;
+  const uint32_t tin_a = ptx::smem_u32(tin0) + (uint32_t)skew * 4u, tout_a = ptx::smem_u32(tout0);
   for (int32_t q = threadIdx.x; q < nunits; q += kThreads) {
     int32_t pl = 0, rem = q;
     if (j.npl > 1) {
@@ -733,6 +752,7 @@ int launch_transform_tile(const float* in, void* out, bool out16, const Geometry
   P.in = in; P.out = out;
   P.status = device_status_word();
   if (!P.status) return IM2WIN_ECUDA;
+  note_transform(1);
   switch (g.Fh) {
     case 1: return launch_tile_fh<1>(P, out16, pl.ctas, pl.smem, st);
     case 2: return launch_tile_fh<2>(P, out16, pl.ctas, pl.smem, st);
@@ -773,6 +793,7 @@ int make_pairs_plan(const Geometry& g, TilePlan* pl) {
   P.H = g.H; P.W = g.W; P.s = g.s; P.Ho = g.Ho; P.L = g.L;
   P.MB = MB; P.nblk = nblk; P.PB = PB;
   P.QW = g.W / 2 + 1;
+  P.test_skip_copy = (knobs().test_skip_copy && ctas == 1) ? 1 : 0;  // (as in the tile plan)
   P.planes = planes; P.HW = hw; P.HoL = g.HoL; P.n_in_total = g.n_in;
   const int64_t units_plane = (int64_t)(nblk == 1 ? g.Ho : MB) * P.QW;
   if (units_plane * PB * units_plane >= ((int64_t)1 << 32)) return IM2WIN_EUNSUPPORTED;  // reciprocal division exact
@@ -805,6 +826,7 @@ int launch_transform_pairs(const float* in, uint16_t* out, const Geometry& g, cu
   pl.P.in = in; pl.P.out = out;
   pl.P.status = device_status_word();
   if (!pl.P.status) return IM2WIN_ECUDA;
+  note_transform(2);
   if (g.Fh == 3) return launch_pairs_fh<3>(pl, st);
   if (g.Fh == 5) return launch_pairs_fh<5>(pl, st);
   if (g.Fh == 7) return launch_pairs_fh<7>(pl, st);
@@ -862,6 +884,7 @@ static int launch_transform_staged(const float* in, float* out, uint16_t* out16,
   if (make_staged_plan(g, &pl) != IM2WIN_OK) {
     const int64_t blocks = (g.n_win + kThreads - 1) / kThreads;
     const int grid = (int)(blocks < 148 * 64 ? blocks : 148 * 64);
+    note_transform(4);
     return out16 ? launch_behind(transform_gather_bf16_kernel, dim3(grid), kThreads, 0, st, in, out16, g.H, g.W, g.Fh, g.s, g.Ho, g.n_win)
                  : launch_behind(transform_gather_kernel, dim3(grid), kThreads, 0, st, in, out, g.H, g.W, g.Fh, g.s, g.Ho, g.n_win);
   }
@@ -882,6 +905,7 @@ static int launch_transform_staged(const float* in, float* out, uint16_t* out16,
   P.magic_Fh = magic_for((uint32_t)g.Fh);
   P.magic_HoL = magic_for((uint32_t)g.HoL);
   const dim3 grid((unsigned)pl.ctas);
+  note_transform(3);
   if (out16) return launch_behind(transform_smem_bf16_kernel, grid, kThreads, smem, st, P, out16);
   return launch_behind(g.Fh == 7 ? transform_smem_kernel<7> : (g.Fh == 11 ? transform_smem_kernel<11> : transform_smem_kernel<0>), grid, kThreads,
                        smem, st, P);

@@ -27,5 +27,7 @@ def test_tile_transform_instantiations_do_not_spill(tmp_path):
     assert sorted(k for k in seen if not k[2]) == [(fh, o, 0) for fh in (1, 2, 3, 4, 5, 7, 11) for o in (0, 1)]
     assert {k[:2]: k[2] for k in seen if k[2]} == columns
     assert all(spill == 0 for spill, _ in seen.values()), seen
+    pairs = [tuple(map(int, v)) for v in re.findall(r"transform_pairs_kernelILi(?:3|5|7|11)E.*?(\d+) bytes spill stores.*?Used (\d+) registers", text, re.S)]
+    assert len(pairs) == 4 and all(spill == 0 and regs <= 40 for spill, regs in pairs), pairs
     # six CTAs of 256 threads per SM (34 KB of shared memory each): at most 40 registers a thread
     assert all(regs <= 40 for (fh, o, form), (_, regs) in seen.items() if fh <= 5 or (fh, o) == (7, 1)), seen
