@@ -656,17 +656,25 @@ int launch_tile_form(const TileParams& P, int64_t ctas, size_t smem, cudaStream_
     cudaGetLastError();
     return IM2WIN_ECUDA;
   }
+  note_transform(1);
   return launch_behind(kern, dim3((unsigned)ctas), kThreads, smem, st, P);
 }
 
+// (bf16 storage under 3, 5, 7 and 11 rows is the pairs kernel's; what that declines and the tile plan takes are tall filters over odd
+// rows, in the column form)
 template <int FH>
 int launch_tile_fh(const TileParams& P, bool out16, int64_t ctas, size_t smem, cudaStream_t st) {
-  if constexpr (FH % 2 == 1 && FH > 1) {
-    if (P.cols)
-      return out16 ? launch_tile_form<FH, true, FH == 3 ? kEither : kColumns>(P, ctas, smem, st)
-                   : launch_tile_form<FH, false, FH == 3 || FH == 11 ? kEither : kColumns>(P, ctas, smem, st);
+  constexpr bool odd = FH % 2 == 1 && FH > 1;
+  if constexpr (odd) {
+    if (P.cols && !out16) return launch_tile_form<FH, false, FH == 3 || FH == 11 ? kEither : kColumns>(P, ctas, smem, st);
+    if constexpr (FH >= 7) {
+      if (P.cols) return launch_tile_form<FH, true, kColumns>(P, ctas, smem, st);
+    }
+    if (out16) return IM2WIN_EUNSUPPORTED;
+  } else {
+    if (out16) return launch_tile_form<FH, true, kQuads>(P, ctas, smem, st);
   }
-  return out16 ? launch_tile_form<FH, true, kQuads>(P, ctas, smem, st) : launch_tile_form<FH, false, kQuads>(P, ctas, smem, st);
+  return launch_tile_form<FH, false, kQuads>(P, ctas, smem, st);
 }
 
 struct TilePlan {
@@ -752,7 +760,6 @@ int launch_transform_tile(const float* in, void* out, bool out16, const Geometry
   P.in = in; P.out = out;
   P.status = device_status_word();
   if (!P.status) return IM2WIN_ECUDA;
-  note_transform(1);
   switch (g.Fh) {
     case 1: return launch_tile_fh<1>(P, out16, pl.ctas, pl.smem, st);
     case 2: return launch_tile_fh<2>(P, out16, pl.ctas, pl.smem, st);

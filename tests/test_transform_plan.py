@@ -146,6 +146,17 @@ def test_every_index_of_the_pairs_transform_stays_in_its_range():
     assert sum(_walk_pairs(shape) for shape in _shapes() if shape[4] in (3, 5, 7, 11)) > 500
 
 
+def test_what_the_pairs_transform_declines():
+    """The column form of tall filters, or the other transforms: no bf16 tile kernel but that is built for these heights."""
+    columns = 0
+    for shape in _shapes() + _far_strides() + [(1, 2, h, w, fh, s) for h in (30, 90, 230) for w in (130, 227, 500, 901) for fh in (5, 7, 11) for s in (1, 2)]:
+        if shape[4] in (3, 5, 7, 11) and not _walk_pairs(shape):
+            form = _walk(shape, 1)
+            assert form is None or (form and shape[4] >= 7)
+            columns += form is not None
+    assert columns > 10
+
+
 def test_strides_far_above_the_filter():
     """What a plan accepts fits shared memory; what it declines is another kernel's."""
     for shape in _far_strides():

@@ -1,5 +1,5 @@
 """What the compiler reports of the tile transform's instantiations: none spills registers, and only filter heights that
-the column form serves (odd, above 1) have it -- beside the quads in one kernel for three rows and for eleven in fp32, else alone -- and the quads' kernels do not."""
+the column form serves (odd, above 1; in bf16 storage 7 and 11, behind the pairs kernel, whose registers are looked at too) have it -- beside the quads in one kernel for three rows and for eleven in fp32, else alone -- and the quads' kernels do not."""
 import os
 import re
 import subprocess
@@ -23,8 +23,8 @@ def test_tile_transform_instantiations_do_not_spill(tmp_path):
         if form:
             spill = int(re.search(r"(\d+) bytes spill stores", body).group(1))
             seen[tuple(int(v) for v in form.groups())] = (spill, int(re.search(r"Used (\d+) registers", body).group(1)))
-    columns = {(3, 0): 2, (3, 1): 2, (5, 0): 1, (5, 1): 1, (7, 0): 1, (7, 1): 1, (11, 0): 2, (11, 1): 1}
-    assert sorted(k for k in seen if not k[2]) == [(fh, o, 0) for fh in (1, 2, 3, 4, 5, 7, 11) for o in (0, 1)]
+    columns = {(3, 0): 2, (5, 0): 1, (7, 0): 1, (7, 1): 1, (11, 0): 2, (11, 1): 1}
+    assert sorted(k for k in seen if not k[2]) == sorted([(fh, 0, 0) for fh in (1, 2, 3, 4, 5, 7, 11)] + [(fh, 1, 0) for fh in (1, 2, 4)])
     assert {k[:2]: k[2] for k in seen if k[2]} == columns
     assert all(spill == 0 for spill, _ in seen.values()), seen
     pairs = [tuple(map(int, v)) for v in re.findall(r"transform_pairs_kernelILi(?:3|5|7|11)E.*?(\d+) bytes spill stores.*?Used (\d+) registers", text, re.S)]
