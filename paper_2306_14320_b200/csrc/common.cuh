@@ -67,7 +67,8 @@ struct Scratch {
 // be the fastest -- for sources no other kernel accepts)
 int launch_conv_tc_strip(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                          Scratch scratch, int src_kind, bool out_bf16, bool even_if_slower = false);
-// Several whole small images per tile of the strip-matrix kernel, where that is the fastest way.
+// Several whole small images per tile of the strip-matrix kernel, where that is the fastest way (the rule, for sources it has scratch for).
+bool strip_images_apply(const Geometry& g, int mode);
 int launch_conv_tc_strip_images(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                                 Scratch scratch, int src_kind, bool out_bf16);
 int launch_conv_tc_persistent(const void* src, const float* f, float* out, const Geometry& g, int mode,

@@ -940,12 +940,14 @@ int launch_conv_tc_strip(const void* src, const float* f, float* out, const Geom
 // transform and convolution 92.7 -> 70.3 us; 69 of 448x6x11, 64 filters, fused 56 -> 31).  Not in TF32 mode (119 calls 1.02), not at
 // stride 2, whose T stages leave the rings too little, and not on deep layers of wide filter tiles whose images are one round of
 // units anyway (32 of 512x9x9, 512 filters, fused: window kernel 45 us, here 51).
+bool strip_images_apply(const Geometry& g, int mode) {
+  if (mode != IM2WIN_MODE_BF16 || g.Fh != 3 || g.Fw != 3 || g.s != 1 || g.N < 2 || (int64_t)g.Ho * g.W > 64) return false;
+  const int64_t n_nt = (g.K + 255) / 256;
+  return !(g.C >= 256 && g.K > 128 * n_nt && g.N * n_nt <= sm_count()) || knobs().strip_images == 1;
+}
 int launch_conv_tc_strip_images(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                                 Scratch scratch, int src_kind, bool out_bf16) {
-  if (out_bf16 || knobs().strip_images == 2) return IM2WIN_EUNSUPPORTED;
-  if (mode != IM2WIN_MODE_BF16 || g.Fh != 3 || g.Fw != 3 || g.s != 1 || g.N < 2 || (int64_t)g.Ho * g.W > 64) return IM2WIN_EUNSUPPORTED;
-  const int64_t n_nt = (g.K + 255) / 256;
-  if (g.C >= 256 && g.K > 128 * n_nt && g.N * n_nt <= sm_count() && knobs().strip_images != 1) return IM2WIN_EUNSUPPORTED;
+  if (out_bf16 || knobs().strip_images == 2 || !strip_images_apply(g, mode)) return IM2WIN_EUNSUPPORTED;
   if (src_kind == 2) return launch_strip<3, 3, 1, true, 2>(src, f, out, g, st, scratch, false, true);
   if (src_kind == 1) return launch_strip<3, 3, 1, true, 1>(src, f, out, g, st, scratch, false, true);
   return launch_strip<3, 3, 1, true, 0>(src, f, out, g, st, scratch, false, true);

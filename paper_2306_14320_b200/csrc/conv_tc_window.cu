@@ -1133,7 +1133,16 @@ bool window_preferred(const Geometry& g, const WParams& P) {
   const int nsm = sm_count();
   if constexpr (kFromInput<SRCK>)
     if (!kPairs<FH, FW> || P.NXS * P.G != g.C) return family_preferred<FH, FW, BF16, SRCK>(g, P);
-  if (SRCK == 3) return xhat_preferred<FH, FW, BF16>(g, P);
+  if constexpr (SRCK == 3) {
+    if (xhat_preferred<FH, FW, BF16>(g, P)) return true;
+    // Also where, from 2e9 multiplications on, this kernel is preferred on the input when the tensor is at hand: with sixteen
+    // channels a source stage at least (longer rows or wider tiles leave it eight), and not where several small images share a
+    // tile of the strip-matrix kernel.  (B200, 1,747 random calls of that size: 64 take this route and 0.84 of the time, 17 -> 11 are slower by
+    // 3 % than a transform and this kernel on the input; 66 images of 16x48x48, 176 5x5 filters, channels-last 121 -> 69 us.)
+    WPlan input;
+    return (double)g.n_out * (double)g.Kg >= 2e9 && !strip_images_apply(g, BF16 ? IM2WIN_MODE_BF16 : IM2WIN_MODE_TF32) &&
+           choose_wplan<FH, FW, BF16, 1>(g, &input) == IM2WIN_OK && input.P.GR >= 16 && window_preferred<FH, FW, BF16, 1>(g, input.P);
+  }
   if (P.units * 2 <= nsm) return false;  // under-filled launches: the persistent kernel's reduction slices
   if (FH == 5) {  // 25 taps of one staged tile (TF32 from the tensor: smaller images)
     if (BF16 || SRCK != 1) return BF16 || P.RPI < 640;
@@ -1271,7 +1280,7 @@ int launch_window(const void* src, const float* f, float* out, const Geometry& g
   if (rc != IM2WIN_OK) return rc;
   note_kernel(KERNEL_WINDOW);
   {
-    const int v[8] = {P.MH + 10 * P.pair + 100 * P.bres, P.G, P.TPS, P.GR, P.SB, P.SR, P.ND, P.box * 100 + P.NBX};
+    const int v[8] = {P.MH + 10 * P.pair + 100 * P.bres + 1000 * SRCK, P.G, P.TPS, P.GR, P.SB, P.SR, P.ND, P.box * 100 + P.NBX};
     note_plan(v, 8);
   }
   return IM2WIN_OK;

@@ -2,6 +2,8 @@
 bit, the result bit for bit on small integers (every product and partial sum is exact), at the edges of tiles: images of less
 than a tile (one contiguous copy per stage), of a tile and a bit, planes that are no whole 16-byte chunks, rows longer than a
 copy box, several filter tiles (each writes the stages of its turn), CTA pairs with an odd number of tiles."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -51,18 +53,33 @@ def test_tensor_and_result(shape, mode):
     assert ran >= 2
 
 
-def test_product_library_takes_it_without_a_transform():
-    """The library's own choice on a layer of the kind it is for, at several batch sizes: tensor and result as above."""
-    apply_config("auto")
-    for n in (8, 33):
-        dims = (n, 64, 30, 30, 64, 3, 3, 1)
-        rng = np.random.default_rng(n)
-        x = rng.integers(-3, 4, dims[:4]).astype(np.float32)
-        f = rng.integers(-3, 4, (64, 64, 3, 3)).astype(np.float32)
-        sh = oracle.Shape(*dims)
-        out, ws = Guarded(n * 64 * 28 * 28), Guarded(b.conv_workspace_bytes(dims, b.SRC_NCHW, b.MODE_TF32) // 4)
-        b.conv(torch.from_numpy(x).cuda(), b.SRC_NCHW, torch.from_numpy(f).cuda(), dims, b.MODE_TF32, out.view, ws.view)
+def _route():
+    """(kernel, source kind of the window-offset kernel, transform kernel) of the last call; clears the last."""
+    plan = (ctypes.c_int * 8)()
+    b.lib().im2win_debug_last_plan(plan)
+    return b.last_kernel(), plan[0] // 1000, b.last_transform()
+
+
+@pytest.mark.parametrize("dims, mode", [
+    ((8, 64, 30, 30, 64, 3, 3, 1), b.MODE_TF32), ((33, 64, 30, 30, 64, 3, 3, 1), b.MODE_TF32),
+    # where it is preferred on the input beside a transform, from 2e9 multiplications on
+    ((66, 16, 48, 48, 176, 5, 5, 1), b.MODE_TF32), ((15, 256, 51, 51, 31, 3, 3, 1), b.MODE_TF32), ((10, 96, 40, 45, 350, 3, 3, 1), b.MODE_BF16),
+], ids=str)
+def test_the_librarys_own_choice_needs_no_transform(dims, mode):
+    n = dims[0]
+    rng = np.random.default_rng(n)
+    few = rng.integers(-3, 4, (2, *dims[1:4])).astype(np.float32)
+    f = rng.integers(-3, 4, (dims[4], dims[1], dims[5], dims[6])).astype(np.float32)
+    sh = oracle.Shape(2, *dims[1:])
+    hat, ref = oracle.im2win(few, sh).reshape(2, -1).view(np.uint32), oracle.conv_direct(few, f, sh).astype(np.float32).reshape(2, -1)
+    x = torch.from_numpy(few).cuda()[torch.arange(n, device="cuda") % 2].contiguous()
+    for config, knobs in (("own choice, test build", {"window_xhat": 0}), ("auto", {})):
+        apply_config(config, **knobs)
+        out, ws = Guarded(n * ref.shape[1]), Guarded((b.conv_workspace_bytes(dims, b.SRC_NCHW, mode) + 3) // 4)
+        if knobs:
+            _route()
+        b.conv(x, b.SRC_NCHW, torch.from_numpy(f).cuda(), dims, mode, out.view, ws.view)
         assert b.last_device_status() == 0
-        hat = oracle.im2win(x, sh).ravel()
-        assert np.array_equal(ws.check()[:hat.size], hat)
-        assert np.array_equal(out.check(), oracle.conv_direct(x, f, sh).astype(np.float32).ravel())
+        assert not knobs or _route() == (b.KERNEL_WINDOW, 3, b.TRANSFORM_NONE)
+        tensor, result = ws.check()[:n * hat.shape[1]].view(np.uint32).reshape(n, -1), out.check().reshape(n, -1)
+        assert all(np.array_equal(tensor[i], hat[i % 2]) and np.array_equal(result[i], ref[i % 2]) for i in range(n))
