@@ -78,12 +78,14 @@ int im2win_workspace_bytes(const im2win_shape* shape, size_t* bytes);
 /* Workspace with which im2win_conv can pick its fastest kernel for (shape, src_kind, mode) (no
  * counterpart in the paper): the im2win tensor where src_kind is NCHW (as above, rounded up to 256
  * bytes), plus room for a re-laid-out copy of the filter that some tensor-core kernels stream by TMA
- * (tap-major orders for the strip-matrix and window-offset kernels, channels completed with zeros; bf16 for BF16 mode; rows padded to the
- * channel groups that do not divide C).  That copy stays below 2 x 4*K'*C'*Fh*Fw bytes, K' the larger of K and 16, C'
+ * (tap-major order for the strip-matrix kernel, images of the filter stages, channels completed with zeros, for the window-offset
+ * kernel; bf16 for BF16 mode; rows padded to the channel groups that do not divide C).  That copy stays below 2 x 4*K'*C'*Fh*Fw bytes, K' the larger of K and 16, C'
  * the larger of C and 32 (most often it is at most the filter's own size), i.e. a few MB against an im2win tensor of tens to hundreds
  * of MB.  A smaller workspace is legal (down to im2win_workspace_bytes, or none for the other source
  * kinds): kernels that need no copy are used instead, some of them slower.  For NCHW_FUSED the size holds no im2win
- * tensor: calls that no fused specialisation takes (see im2win_conv) want im2win_workspace_bytes where that is more. */
+ * tensor: calls that no fused specialisation takes (see im2win_conv) want im2win_workspace_bytes where that is more, and so do
+ * layers of stride 1 with filters other than 3x3 and 5x5, or whose channels are no multiple of 16 (TF32) or 32 (BF16): the
+ * window-offset kernel, often the fastest on those, takes them where the workspace has room for the tensor. */
 int im2win_conv_workspace_bytes(const im2win_shape* shape, int src_kind, int mode, size_t* bytes);
 
 /* Bytes an im2col matrix for the whole batch would take, 4*N*C*Fh*Fw*Ho*Wo (Section III-A).

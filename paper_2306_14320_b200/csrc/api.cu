@@ -96,10 +96,10 @@ int launch_conv_tc(const void* src, const float* f, float* out, const Geometry& 
   return IM2WIN_EUNSUPPORTED;
 }
 
-size_t conv_scratch_bytes(const Geometry& g, int mode, int src_kind) {
+size_t conv_scratch_bytes(const Geometry& g, int mode, int src_kind, bool window) {
   if (mode != IM2WIN_MODE_TF32 && mode != IM2WIN_MODE_BF16) return 0;
   const size_t a = strip_scratch_bytes(g, mode, src_kind), b = persistent_scratch_bytes(g, mode);
-  const size_t c = knobs().no_window ? 0 : window_scratch_bytes(g, mode, src_kind);
+  const size_t c = knobs().no_window || !window ? 0 : window_scratch_bytes(g, mode, src_kind);
   return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
@@ -363,7 +363,9 @@ int im2win_conv_workspace_bytes(const im2win_shape* shape, int src_kind, int mod
   if (mode != IM2WIN_MODE_TF32 && mode != IM2WIN_MODE_BF16 && mode != IM2WIN_MODE_FP32) return IM2WIN_EINVAL;
   const size_t win = src_kind == IM2WIN_SRC_NCHW ? ((size_t)g.n_win * 4 + 255) / 256 * 256 : 0;
   const int kind = src_kind == IM2WIN_SRC_NCHW_FUSED ? 1 : (src_kind == IM2WIN_SRC_IM2WIN_BF16 ? 2 : 0);
-  size_t extra = conv_scratch_bytes(g, mode, kind);
+  // (fused calls of the window-offset kernel's wider families take that kernel only with room for the im2win tensor: without it
+  // they would pay for a copy that no kernel reads)
+  size_t extra = conv_scratch_bytes(g, mode, kind, /*window=*/!(kind == 1 && window_family(g, mode)));
   if (src_kind == IM2WIN_SRC_NCHW) {  // (the window-offset kernel that writes the tensor itself)
     const size_t own = window_scratch_bytes(g, mode, 3);
     if (own > extra) extra = own;

@@ -97,7 +97,7 @@ double gather_us(const Geometry& g, int mode);
 bool gather_beats_transform(const Geometry& g, int mode);
 int launch_conv_tc_gather(const float* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                           bool fused, bool behind_transform);
-size_t conv_scratch_bytes(const Geometry& g, int mode, int src_kind);
+size_t conv_scratch_bytes(const Geometry& g, int mode, int src_kind, bool window = true);
 // Shared body of im2win_conv / im2win_conv_bf16out / im2win_conv_static (argument checks, workspace
 // split into the im2win tensor and the filter scratch, transform, dispatch).
 int conv_impl(const void* src, int src_kind, const float* filter, const im2win_shape* shape, int mode, void* out,
