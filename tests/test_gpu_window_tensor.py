@@ -53,6 +53,23 @@ def test_tensor_and_result(shape, mode):
     assert ran >= 2
 
 
+def test_product_library_takes_it_without_a_transform():
+    """The library's own choice on a layer of the kind it is for, at several batch sizes: tensor and result as above."""
+    apply_config("auto")
+    for n in (8, 33):
+        dims = (n, 64, 30, 30, 64, 3, 3, 1)
+        rng = np.random.default_rng(n)
+        x = rng.integers(-3, 4, dims[:4]).astype(np.float32)
+        f = rng.integers(-3, 4, (64, 64, 3, 3)).astype(np.float32)
+        sh = oracle.Shape(*dims)
+        out, ws = Guarded(n * 64 * 28 * 28), Guarded(b.conv_workspace_bytes(dims, b.SRC_NCHW, b.MODE_TF32) // 4)
+        b.conv(torch.from_numpy(x).cuda(), b.SRC_NCHW, torch.from_numpy(f).cuda(), dims, b.MODE_TF32, out.view, ws.view)
+        assert b.last_device_status() == 0
+        hat = oracle.im2win(x, sh).ravel()
+        assert np.array_equal(ws.check()[:hat.size], hat)
+        assert np.array_equal(out.check(), oracle.conv_direct(x, f, sh).astype(np.float32).ravel())
+
+
 def _route():
     """(kernel, source kind of the window-offset kernel, transform kernel) of the last call; clears the last."""
     plan = (ctypes.c_int * 8)()
