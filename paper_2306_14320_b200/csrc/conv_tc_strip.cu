@@ -940,10 +940,20 @@ int launch_conv_tc_strip(const void* src, const float* f, float* out, const Geom
 // transform and convolution 92.7 -> 70.3 us; 69 of 448x6x11, 64 filters, fused 56 -> 31).  Not in TF32 mode (119 calls 1.02), not at
 // stride 2, whose T stages leave the rings too little, and not on deep layers of wide filter tiles whose images are one round of
 // units anyway (32 of 512x9x9, 512 filters, fused: window kernel 45 us, here 51).
+// Nor, in NCHW order, where 32 or 64 channels (one or two T stages) leave a unit little to overlap its turn-around with and there are
+// several rounds of them: against the persistent kernel, whose tiles hold no rows that are dropped, 32 channels want as many rounds as
+// that kernel and no more than two, 64 no more than two or fewer than twice as many.  (B200, 1,589 random calls of this kernel, half of
+// them of 32 channels: 332 go back to the other kernels, slower by more than 3 % than before this kernel took several images 172 -> 13;
+// 302 images of 18x4, 704 filters, fused 40 -> 23 us.  Channels-last 2 of 395 are slower: the others store that order worse.)
 bool strip_images_apply(const Geometry& g, int mode) {
   if (mode != IM2WIN_MODE_BF16 || g.Fh != 3 || g.Fw != 3 || g.s != 1 || g.N < 2 || (int64_t)g.Ho * g.W > 64) return false;
-  const int64_t n_nt = (g.K + 255) / 256;
-  return !(g.C >= 256 && g.K > 128 * n_nt && g.N * n_nt <= sm_count()) || knobs().strip_images == 1;
+  if (knobs().strip_images == 1) return true;
+  const int64_t n_nt = (g.K + 255) / 256, nsm = sm_count();
+  if (g.C >= 256 && g.K > 128 * n_nt && g.N * n_nt <= nsm) return false;
+  if (g.C > 64 || g.out_nhwc) return true;
+  const int64_t ipt = 128 / ((int64_t)g.Ho * g.W) < g.N ? 128 / ((int64_t)g.Ho * g.W) : g.N;
+  const int64_t rounds = ((g.N + ipt - 1) / ipt * n_nt + nsm - 1) / nsm, packed = ((g.Mtot + 127) / 128 * n_nt + nsm - 1) / nsm;
+  return g.C <= 32 ? rounds <= 2 && rounds <= packed : rounds <= 2 || rounds < 2 * packed;
 }
 int launch_conv_tc_strip_images(const void* src, const float* f, float* out, const Geometry& g, int mode, cudaStream_t st,
                                 Scratch scratch, int src_kind, bool out_bf16) {
