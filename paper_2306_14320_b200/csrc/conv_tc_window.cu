@@ -1073,7 +1073,9 @@ bool xhat_preferred(const Geometry& g, const WParams& P) {
 // against the persistent kernel (behind the transform for kind 3) and, where that would be taken, the gather kernel, all in
 // microseconds.  Fits to 3,100 random calls on B200 (this kernel within 10 % in the median, the persistent kernel within 18 %).
 // Over those calls the picks take 0.86 of the others' time from SRC_NCHW and 0.94 fused, the better of the two on each 0.80 and
-// 0.88; 79 of them are slower than the others by more than 3 %.  Filters without a persistent kernel (3x4) are compared with the
+// 0.88; 79 of them are slower than the others by more than 3 %.  Channels-last with one accumulator the picks were slower the more
+// rounds there are: of 513 such picks 112 go back to the others, those slower than them by more than 3 % fall from 71 to 47 (71 images of
+// 17x75x44, 176 1x3 filters, BF16 84 -> 70 us; 28 of 39x97x73, 208 3x3 filters 129 -> 107).  Filters without a persistent kernel (3x4) are compared with the
 // gather kernel alone: 0.66 and 0.75, none slower.  (77 images of 64x53x58, 80 3x4 filters, BF16 325 -> 74 us; 39 of 160x22x16, 176
 // 1x7 filters, channels-last 28.5 -> 16.5; 59 of 75x22x22, 48 5x5 filters, fused 46 -> 21.)
 template <int FH, int FW, bool BF16, int SRCK>
@@ -1087,6 +1089,9 @@ bool family_preferred(const Geometry& g, const WParams& P) {
   constexpr bool XHAT = SRCK == 3;
   const double *a = on[XHAT][BF16], *o = off[XHAT][BF16];
   if (g.C < 16) return false;
+  // (one filter row: few MMAs a stage, and two source stages of eight channels, from which the tensor is written too, do not keep up
+  // with many channels.  Channels-last, 18 images of 416x29x15, 480 1x3 filters, TF32 53 us here, 38 the others; up to 82 channels on a par)
+  if (XHAT && FH == 1 && P.nhwc && P.GR == 8 && P.SR == 2 && g.C > 128) return false;
   const int64_t nsm = sm_count(), slots = P.pair ? nsm / 2 : nsm, rounds = (P.units + slots - 1) / slots, step = BF16 ? 16 : 8;
   const double mma = FH * FW * (double)(P.NXS * P.G / step) * P.MH * (P.NT > 108 ? P.NT / 2.0 : 54.0) / 1900.0;
   const double extra = XHAT ? g.C * 128 * P.MH * FH * 4 / P.n_ntiles * 1e-5 : (P.nhwc ? P.NT * P.MH * 0.01 : 0.0);
@@ -1105,7 +1110,9 @@ bool family_preferred(const Geometry& g, const WParams& P) {
     const bool resident = P.n_ntiles == 1 && ng * S * P.NT * 32 < 150000;
     there = o[0] + o[1] * bytes + o[2] * steps + (resident ? 0.0 : o[3] * steps * P.NT * 0.01) +
             o[4] * (double)waves * P.NT * 0.01 * (P.nhwc ? 2.0 : 1.0) + (z > 1 ? o[5] : 0.0);
-    if (here >= 0.9 * there) return false;
+    // (channels-last columns behind one accumulator: every round but the last holds up the next round's MMAs for longer than the fit says)
+    const double exposed = P.nhwc && P.ND == 1 ? 1.25 * (double)(rounds - 1) * P.NT * P.MH * 0.01 : 0.0;
+    if (here + exposed >= 0.9 * there) return false;
   }
   const int mode = BF16 ? IM2WIN_MODE_BF16 : IM2WIN_MODE_TF32;
   if ((FH == 3 && FW == 4) || gather_preferred(g, mode, true)) {
