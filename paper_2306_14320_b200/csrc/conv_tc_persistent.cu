@@ -523,7 +523,8 @@ conv_tc_persistent_kernel(const PParams P, const __grid_constant__ CUtensorMap f
     // The kernel is launched as a programmatic dependent of whatever precedes it in the stream: where that is
     // the transform kernel (which lets its dependents start while it drains), the prologue above overlapped
     // its tail, and the source is read only once that grid has completed.  After any other kernel: no effect.
-    // (Behind this call's own filter-copy kernel, an ordinary launch, everything earlier has completed already.)
+    // (Behind this call's own filter-copy kernel everything earlier has completed already: that grid waits for it before it lets
+    // this one start, ptx::pdl_enter.)
     if (P.wait_prev) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (P.box) {
       // One 2-D box per channel group.  The tile lies in one image: x = first needed float of the
@@ -1519,7 +1520,8 @@ int launch_spec_impl(const void* xhat, const float* f, float* out, const Geometr
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  // (the filter copy itself is an ordinary launch: when it runs, everything before it has completed)
+  // (the filter copy begins with ptx::pdl_enter: it waits for everything before it, and only then lets this kernel start.  The other
+  // way round, source reads and output writes here could run beside the kernels before it.)
   P.wait_prev = f_copy ? 0 : 1;
   if (resident) {
     auto kern = conv_tc_persistent_kernel<FH, FW, CB, BF16, true, FUSED, SRC16, OUT16>;

@@ -1042,8 +1042,8 @@ double persistent_fused_us(const Geometry& g, const WParams& P) {
 // both in microseconds: fits to 1,200 random calls on B200 (this kernel within 9 % in the median, the others within 13 %).
 // Over those calls the picks take 0.89 of the others' time, the better of the two on each 0.85; where this kernel is not
 // expected to win by a fourteenth the others stay (1 in a hundred picks is more than 3 % slower than them).
-// (128 images of 64x58x58, 64 filters, TF32 166 -> 124 us a call with new inputs; 32 of 384x15x15, 384 filters 60 -> 54; 119 of
-// 128x58x58, 85 filters, BF16 267 -> 191.)
+// (128 images of 64x58x58, 64 filters, TF32 169 -> 127 us a call, the first on new buffers 193 -> 161; 32 of 384x15x15, 384
+// filters 60 -> 51, 75 -> 71; 119 of 128x58x58, 85 filters, BF16 267 -> 191.)
 template <int FH, int FW, bool BF16>
 bool xhat_preferred(const Geometry& g, const WParams& P) {
   //                                     start  MMAs   rows  columns tensor  pairs
@@ -1074,10 +1074,11 @@ bool xhat_preferred(const Geometry& g, const WParams& P) {
 // microseconds.  Fits to 3,100 random calls on B200 (this kernel within 10 % in the median, the persistent kernel within 18 %).
 // Over those calls the picks take 0.86 of the others' time from SRC_NCHW and 0.94 fused, the better of the two on each 0.80 and
 // 0.88; 79 of them are slower than the others by more than 3 %.  Channels-last with one accumulator the picks were slower the more
-// rounds there are: of 513 such picks 112 go back to the others, those slower than them by more than 3 % fall from 71 to 47 (71 images of
-// 17x75x44, 176 1x3 filters, BF16 84 -> 70 us; 28 of 39x97x73, 208 3x3 filters 129 -> 107).  Filters without a persistent kernel (3x4) are compared with the
-// gather kernel alone: 0.66 and 0.75, none slower.  (77 images of 64x53x58, 80 3x4 filters, BF16 325 -> 74 us; 39 of 160x22x16, 176
-// 1x7 filters, channels-last 28.5 -> 16.5; 59 of 75x22x22, 48 5x5 filters, fused 46 -> 21.)
+// rounds there are: of 513 such picks 112 go back to the others, those slower by more than 3 % than before this kernel took them
+// fall from 53 to 9 (71 images of 17x75x44, 176 1x3 filters, BF16 84 -> 70 us; 28 of 39x97x73, 208 3x3 filters 129 -> 107).  Filters
+// without a persistent kernel (3x4) are compared with the gather kernel alone: 0.66 and 0.75, none slower.  (77 images of
+// 64x53x58, 80 3x4 filters, BF16 325 -> 74 us; 39 of 160x22x16, 176 1x7 filters, channels-last 28.5 -> 16.5; 59 of 75x22x22, 48 5x5
+// filters, fused 46 -> 21.)
 template <int FH, int FW, bool BF16, int SRCK>
 bool family_preferred(const Geometry& g, const WParams& P) {
   //                                     start  MMAs   rows  columns tensor / channels-last columns  pairs
